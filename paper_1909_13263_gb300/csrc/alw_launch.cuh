@@ -16,7 +16,7 @@ static int launch_one(const StageParams &p, cudaStream_t stream) {
     configured = true;
   }
   dim3 grid(p.tiles_x, p.tiles_y);
-  kern<<<grid, Sh::NT, smem, stream>>>(p);
+  kern<<<grid, Sh::NT, smem, stream>>>(p, sweep_args<PREC, W>(p));
   return (int)cudaGetLastError();
 }
 

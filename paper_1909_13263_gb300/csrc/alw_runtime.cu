@@ -113,7 +113,7 @@ void alw::dev_free(void *ptr, size_t bytes, void *stream) {
 }
 
 int alw::tile_x(int prec, int dim) {
-  if (dim == 1) return TX1D;
+  if (dim == 1) return prec == P_F64 ? TX1D64 : TX1D;
   return prec == P_F64 ? Tile<P_F64>::TX : Tile<P_F32>::TX;
 }
 int alw::tile_y(int prec, int dim) {

@@ -1,8 +1,108 @@
 // The fused RK-stage kernel (see alw_device.cuh for the arithmetic).
 #pragma once
+#include <type_traits>
+
 #include "alw_device.cuh"
+#include "alw_sweep64.cuh"
 
 namespace alw {
+
+// Constants of the FP64 sweeps, formed on the host (nothing for the float variants).
+template <int PREC> struct SweepArgs {};
+template <> struct SweepArgs<P_F64> {
+  Sweep64 x, y;
+};
+template <int PREC, int W>
+static SweepArgs<PREC> sweep_args(const StageParams &p) {
+  SweepArgs<PREC> a;
+  if constexpr (PREC == P_F64) {
+    a.x = make_sweep64<W>(p.dx, p.eps);
+    a.y = p.dim == 2 ? make_sweep64<W>(p.dy, p.eps) : a.x;
+  }
+  return a;
+}
+
+// Largest of two non-negative doubles by their bit patterns (integer comparisons: FP64 ones run on the FP64
+// pipe); a NaN counts as larger than everything, so it survives to the caller's check.
+__device__ __forceinline__ double max_bits(double a, double b) {
+  const unsigned long long x = double_to_bits(a), y = double_to_bits(b);
+  return bits_to_double(x > y ? x : y);
+}
+__device__ __forceinline__ double min_bits(double a, double b) {
+  const unsigned long long x = double_to_bits(a), y = double_to_bits(b);
+  return bits_to_double(x < y ? x : y);
+}
+
+// H at the mean one-sided derivatives and the node alpha in double, sharing what they have in common.
+// With c = (u^- + u^+ + v^- + v^+)/2 and e = (|u^+ - u^-| + |v^+ - v^-|)/2 the four corner sums u + v are
+// c +- e and c +- |du - dv|/2.  `known` is a lower bound of the grid maximum the alphas are folded into:
+// an alpha that cannot exceed it is returned as 0 (0 = evaluate always, for a flux that uses the node's own).
+// The trigonometric kinds need sin and cos of c only: |cos(c +- d)| is at most |cos c| cos d + |sin c| sin d,
+// attained by one of the two signs, with cos d and sin d by their series for small d.
+__device__ __forceinline__ void ham_node64(int kind, double um, double up, double vm, double vp, double x, double y,
+                                           double known, double &H, double &ax, double &ay) {
+  const double su = up + um, du = up - um;
+  switch (kind) {
+    case H_BURGERS2D:
+    case H_BURGERS1D: {
+      const bool two = kind == H_BURGERS2D;
+      const double c = fma(0.5, two ? su + (vp + vm) : su, 1.0);
+      H = 0.5 * c * c;
+      ax = fma(0.5, two ? fabs(du) + fabs(vp - vm) : fabs(du), fabs(c));
+      ay = two ? ax : 0.0;
+    } break;
+    case H_NEGCOS2D:
+    case H_NEGCOS1D:
+    case H_SIN2D: {
+      const bool two = kind != H_NEGCOS1D;
+      const double s2 = two ? su + (vp + vm) : su;
+      const double c = kind == H_SIN2D ? 0.5 * s2 : fma(0.5, s2, 1.0);
+      double sn, cs;
+      sincos(c, &sn, &cs);
+      H = kind == H_SIN2D ? sn : -cs;
+      const double a = fabs(kind == H_SIN2D ? cs : sn), b = fabs(kind == H_SIN2D ? sn : cs);
+      const double dv = two ? vp - vm : 0.0;
+      const double e = 0.5 * (fabs(du) + fabs(dv));
+      ax = 0.0;
+      if (!(fma(b, e, a) <= known)) {
+        const double e2 = 0.5 * fabs(fabs(du) - fabs(dv));
+        auto corner = [&](double d) {
+          double sd, cd;
+          if (d <= 0.015625) {
+            const double q = d * d;
+            cd = fma(q, fma(q, fma(q, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
+            sd = d * fma(q, fma(q, 1.0 / 120.0, -1.0 / 6.0), 1.0);
+            return fma(a, cd, b * sd);
+          }
+          sincos(c + d, &sn, &cs);
+          const double r1 = fabs(kind == H_SIN2D ? cs : sn);
+          sincos(c - d, &sn, &cs);
+          return max_bits(r1, fabs(kind == H_SIN2D ? cs : sn));
+        };
+        ax = corner(e);
+        if (two) ax = max_bits(ax, corner(e2));
+      }
+      ay = two ? ax : 0.0;
+    } break;
+    case H_ADVECT1D: {
+      H = 0.5 * su;
+      ax = fabs(su) < INFINITY ? 1.0 : NAN;
+      ay = 0.0;
+    } break;
+    case H_EIKONAL2D: {
+      const double p = 0.5 * su, q = 0.5 * (vp + vm);
+      H = sqrt(fma(p, p, fma(q, q, 1.0)));
+      // |H_p| = |u| / sqrt(u^2 + v^2 + 1) grows with |u| and falls with |v|
+      const double ul = min_bits(fabs(um), fabs(up)), uh = max_bits(fabs(um), fabs(up));
+      const double vl = min_bits(fabs(vm), fabs(vp)), vh = max_bits(fabs(vm), fabs(vp));
+      ax = uh * rsqrt(fma(uh, uh, fma(vl, vl, 1.0)));
+      ay = vh * rsqrt(fma(vh, vh, fma(ul, ul, 1.0)));
+    } break;
+    default:
+      H = ham_value<double>(kind, 0.5 * su, 0.5 * (vp + vm), x, y);
+      node_alpha<double>(kind, um, up, vm, vp, x, y, ax, ay);
+  }
+}
 
 template <int PREC> struct Types;
 template <> struct Types<P_F64> { using S = double; using C = double; };
@@ -13,10 +113,11 @@ template <> struct Types<P_MIXED> { using S = float; using C = float; };
 // sweep segments (SMALL = 1), or 2-node segments (SMALL = 2: twice the threads per tile, for grids
 // whose 16 x 16 tiles are fewer than the SMs).
 template <int PREC, int DIM, int SMALL = 0> struct Shape {
-  static constexpr int TX = (DIM == 2) ? (SMALL ? 16 : Tile<PREC>::TX) : TX1D;
+  static constexpr int TX = (DIM == 2) ? (SMALL ? 16 : Tile<PREC>::TX) : (PREC == P_F64 ? TX1D64 : TX1D);
   static constexpr int TY = (DIM == 2) ? (SMALL ? 16 : Tile<PREC>::TY) : 1;
-  static constexpr int K = (DIM == 2) ? (SMALL == 2 ? 2 : SMALL == 1 ? 4 : Tile<PREC>::K) : K1D;
+  static constexpr int K = (DIM == 2) ? (SMALL == 2 ? 2 : SMALL == 1 ? 4 : Tile<PREC>::K) : (PREC == P_F64 ? 1 : K1D);
   static constexpr int NT = (TX / K) * TY;          // threads per CTA
+  static constexpr int MINB = (PREC == P_F64 && DIM == 2) ? 512 / NT : 1;   // FP64: 16 warps per SM
   static constexpr int SW = TX + 8;                 // smem row: GX halo on each side
   static constexpr int SH = (DIM == 2) ? TY + 6 : 1;
   static constexpr int NARR = (PREC == P_MIXED) ? 3 : 1;
@@ -26,8 +127,25 @@ template <int PREC, int DIM, int SMALL = 0> struct Shape {
   }
 };
 
+// FP64: one-sided derivatives of K consecutive nodes from the cells a, a + step, ... (a = first node - 3) with
+// the weights in float pairs; nv nodes of the segment count.  False when the segment does not qualify (and
+// for the float variants).
+template <int PREC, int K, int W, class S, class C>
+__device__ __forceinline__ bool sweep_pairs(const S *a, int step, const SweepArgs<PREC> &sw, bool along_y, int nv,
+                                            C (&dm)[K], C (&dp)[K]) {
+  if constexpr (PREC == P_F64) {
+    return sweep64<K, W>([&](int m) { return a[m * step]; }, along_y ? sw.y : sw.x, nv, [&](int q, double x, double y) {
+      dm[q] = x;
+      dp[q] = y;
+    });
+  } else {
+    return false;
+  }
+}
+
 template <int PREC, int DIM, int WEIGHTS, int SMALL>
-__global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT) stage_kernel(const StageParams p) {
+__global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT, Shape<PREC, DIM, SMALL>::MINB)
+    stage_kernel(const StageParams p, const SweepArgs<PREC> sw) {
   using S = typename Types<PREC>::S;
   using C = typename Types<PREC>::C;
   using Sh = Shape<PREC, DIM, SMALL>;
@@ -114,20 +232,33 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT) stage_kernel(cons
 
   C amx = C(0), amy = C(0);
   bool bad = false;
+  if constexpr (PREC == P_F64) {
+    // what other CTAs have folded so far is a lower bound of the grid maximum
+    if (!local_alpha && p.write_slot >= 0) {
+      amx = bits_to_double(*(volatile unsigned long long *)&st->alpha_bits[p.write_slot][0]);
+      amy = bits_to_double(*(volatile unsigned long long *)&st->alpha_bits[p.write_slot][1]);
+    }
+  }
 
   // RK combination, store, and alpha bookkeeping for node (lx, ly) of the tile
   auto finish_node = [&](int lxn, int lyn, C um, C up, C vm, C vp) {
     const int gi = tx0 + lxn, gj = ty0 + lyn;
     if (gi >= p.nx || gj >= p.ny) return;
-    C ax, ay;
+    C ax, ay, H;
     const C xn = C(p.xlo + gi * p.dx), yn = C(p.ylo + gj * p.dy);
-    node_alpha<C>(p.ham, um, up, vm, vp, xn, yn, ax, ay);
-    if (!(isfinite(ax) && isfinite(ay))) bad = true;
-    amx = fmax(amx, ax);
-    amy = fmax(amy, ay);
+    if constexpr (PREC == P_F64) {
+      ham_node64(p.ham, um, up, vm, vp, xn, yn, local_alpha ? -1.0 : (amx < amy ? amx : amy), H, ax, ay);
+      amx = max_bits(amx, ax);
+      amy = max_bits(amy, ay);
+    } else {
+      node_alpha<C>(p.ham, um, up, vm, vp, xn, yn, ax, ay);
+      H = ham_value<C>(p.ham, C(0.5) * (up + um), C(0.5) * (vp + vm), xn, yn);
+      if (!(isfinite(ax) && isfinite(ay))) bad = true;
+      amx = fmax(amx, ax);
+      amy = fmax(amy, ay);
+    }
     if (p.stage == 0) return;
     const C aX = local_alpha ? ax : fax, aY = local_alpha ? ay : fay;
-    const C H = ham_value<C>(p.ham, C(0.5) * (up + um), C(0.5) * (vp + vm), xn, yn);
     const C L = -((H - aX * C(0.5) * (up - um)) - aY * C(0.5) * (vp - vm));
     const int sidx = ((DIM == 2) ? lyn + 3 : 0) * SW + lxn + 4;
     if (PREC == P_MIXED) {
@@ -156,11 +287,18 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT) stage_kernel(cons
         const size_t g = (size_t)(gj + ((DIM == 2) ? GY : 0)) * p.pitch + gi + GX;
         const C base = C(reinterpret_cast<const S *>(p.base0)[g]);
         if (p.stage == 2) outv = C(0.75) * base + C(0.25) * (src + C(dt) * L);
-        else outv = base / C(3) + C(2) * (src + C(dt) * L) / C(3);
+        else if (PREC == P_F64) {
+          // (phi^n + 2 (phi_2 + dt L)) / 3, the division as a product with its remainder folded back
+          const C z = fma(C(2), fma(C(dt), L, src), base), third = C(1) / C(3), q = z * third;
+          outv = fma(fma(C(-3), q, z), third, q);
+        } else outv = base / C(3) + C(2) * (src + C(dt) * L) / C(3);
       }
       store_node<S, DIM>(reinterpret_cast<S *>(p.out0), p.pitch, p.nx, p.ny, p.bc, gi, gj, S(outv));
     }
   };
+
+  // nodes of a K-node segment that lie inside the grid
+  auto valid = [&](int left, bool inside) { return !inside || left <= 0 ? -9 : (left < K ? left : K); };
 
   // ---- phase X: each thread sweeps K consecutive nodes of one row
   {
@@ -168,11 +306,14 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT) stage_kernel(cons
     const int r = tid / SEGS, seg = tid - r * SEGS;
     const int srow = (DIM == 2) ? r + 3 : 0;
     const int base_i = srow * SW + seg * K + 1;     // smem index of node x = seg*K - 3
-    C v[K + 5];
-#pragma unroll
-    for (int m = 0; m < K + 5; ++m) v[m] = diff(base_i + m, base_i + m + 1, rdx);
     C dm[K], dp[K];
-    weno_sweep<C, K, WEIGHTS>(v, rdx, dx, eps, dm, dp);
+    const int nv = valid(p.nx - tx0 - seg * K, DIM == 1 || ty0 + r < p.ny);
+    if (!sweep_pairs<PREC, K, WEIGHTS>(s_a + base_i, 1, sw, false, nv, dm, dp)) {
+      C v[K + 5];
+#pragma unroll
+      for (int m = 0; m < K + 5; ++m) v[m] = diff(base_i + m, base_i + m + 1, rdx);
+      weno_sweep<C, K, WEIGHTS>(v, rdx, dx, eps, dm, dp);
+    }
     if (DIM == 2) {
 #pragma unroll
       for (int q = 0; q < K; ++q) {
@@ -190,11 +331,14 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT) stage_kernel(cons
     const int x = tid % TX, seg = tid / TX;
     const int col = x + 4;
     const C dy = C(p.dy), rdy = C(p.rdy);
-    C v[K + 5];
-#pragma unroll
-    for (int m = 0; m < K + 5; ++m) v[m] = diff((seg * K + m) * SW + col, (seg * K + m + 1) * SW + col, rdy);
     C vm[K], vp[K];
-    weno_sweep<C, K, WEIGHTS>(v, rdy, dy, eps, vm, vp);
+    const int nv = valid(p.ny - ty0 - seg * K, tx0 + x < p.nx);
+    if (!sweep_pairs<PREC, K, WEIGHTS>(s_a + seg * K * SW + col, SW, sw, true, nv, vm, vp)) {
+      C v[K + 5];
+#pragma unroll
+      for (int m = 0; m < K + 5; ++m) v[m] = diff((seg * K + m) * SW + col, (seg * K + m + 1) * SW + col, rdy);
+      weno_sweep<C, K, WEIGHTS>(v, rdy, dy, eps, vm, vp);
+    }
 #pragma unroll
     for (int q = 0; q < K; ++q) {
       const int y = seg * K + q;
@@ -204,10 +348,15 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT) stage_kernel(cons
 
   // ---- grid maximum of alpha: warp shuffle, then one atomicMax per CTA
   double mx = double(amx), my = double(amy);
+  if (PREC == P_F64) {
+    // a NaN or an infinity in any alpha is the thread's maximum
+    bad = !(mx < INFINITY) || !(my < INFINITY);
+    if (bad) mx = my = 0.0;
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    my = fmax(my, __shfl_xor_sync(0xffffffffu, my, o));
+    mx = max_bits(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    my = max_bits(my, __shfl_xor_sync(0xffffffffu, my, o));
   }
   const int anybad = __syncthreads_or(bad ? 1 : 0);
   if ((tid & 31) == 0) {
@@ -217,8 +366,8 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT) stage_kernel(cons
   __syncthreads();
   if (tid == 0) {
     for (int w = 1; w < NT / 32; ++w) {
-      mx = fmax(mx, s_red[0][w]);
-      my = fmax(my, s_red[1][w]);
+      mx = max_bits(mx, s_red[0][w]);
+      my = max_bits(my, s_red[1][w]);
     }
     if (anybad) atomicOr(&st->err, 1);
     if (p.write_slot >= 0) {

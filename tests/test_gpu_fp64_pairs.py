@@ -1,0 +1,79 @@
+"""FP64 stages whose nonlinear weights are formed in float pairs, against the FP64 oracle.
+
+On smooth data every segment qualifies for the pairs.  Kernel and oracle then differ by rounding only: a
+stage rounds phi + dt L once (half a unit of the largest |phi|, u = 2^-53) after three or four rounded
+operations of the same size, and L's own error, a few u of |phi_x|, enters times dt |H_p| <= 0.6 dx; the
+bound is 16 u of max |phi|.  Data with kinks, noise or an offset mix qualifying and other segments; there
+the indicators of single-precision size are amplified as in test_gpu_parity.py (1e-12).
+"""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+from gpucase import Case, oracle_stages, rel_err
+from paper_1909_13263_gb300 import inputs, native
+
+pytestmark = pytest.mark.gpu
+
+SMOOTH_TOL = 16 * 2.0**-53
+FP64_TOL = 1e-12
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    native.load()
+    native.use_torch_allocator(True)
+    yield
+
+
+def _errors(case, phi0):
+    a, _ = oracle.alpha_of(case.cfg(), phi0)
+    dt = 0.6 / (a[0] / case.dx + (a[1] / case.dy if case.dim == 2 else 0.0))
+    ref = oracle_stages(case, phi0, dt)
+    with case.solver() as s:
+        s.set_phi0(phi0)
+        errs = []
+        for stage in (1, 2, 3):
+            s.run_stage(stage, dt)
+            errs.append(rel_err(s.get_stage_phi(stage) if stage < 3 else s.get_phi(), ref[stage - 1]))
+    return errs
+
+
+def _smooth(case):
+    # one wave over the domain, resolved by the smallest of the grids below
+    x, _ = inputs.axis(case.nx, case.lo, case.hi, case.bc)
+    if case.dim == 1:
+        return -np.cos(np.pi * x + 0.3)
+    y, _ = inputs.axis(case.ny, case.lo, case.hi, case.bc)
+    return -np.cos(np.pi * (x[None, :] + 2.0 * y[:, None]) / 2.0 + 0.3)
+
+
+# edges of the 16 x 16 and 32 x 16 tiles and of the 1D tiles, ragged and rectangular
+@pytest.mark.parametrize("weights", ["arclength", "jp"])
+@pytest.mark.parametrize("shape", [(2, 31, 33), (2, 64, 48), (2, 161, 163), (2, 1025, 130), (1, 63, 1), (1, 64, 1),
+                                   (1, 65, 1), (1, 321, 1), (1, 5000, 1)], ids=str)
+def test_smooth_stages_match_oracle_to_rounding(shape, weights):
+    dim, nx, ny = shape
+    case = Case(dim, nx, ny, "negcos2d" if dim == 2 else "burgers1d", weights=weights, lo=-2.0 if dim == 2 else -1.0,
+                hi=2.0 if dim == 2 else 1.0, alpha_mode="global_lagged" if dim == 2 else "local_lagged")
+    assert max(_errors(case, _smooth(case))) <= SMOOTH_TOL
+
+
+@pytest.mark.parametrize("weights", ["arclength", "jp"])
+@pytest.mark.parametrize("kind", ["kinks", "noise", "offset", "huge", "tiny"])
+def test_mixed_segments_match_oracle(kind, weights):
+    case = Case(2, 97, 75, "sin2d", bc="linextrap", weights=weights)
+    x, _ = inputs.axis(97, -1.0, 1.0, "linextrap")
+    y, _ = inputs.axis(75, -1.0, 1.0, "linextrap")
+    phi0 = math.pi * (np.abs(y[:, None] - 0.03) - np.abs(x[None, :] + 0.01))
+    if kind == "noise":
+        phi0[20:30, 40:60] += 0.01 * inputs.random_field(10, 20, 3, "rough")
+    elif kind == "offset":
+        phi0 = 1e3 + np.sin(2.0 * x[None, :] + y[:, None])
+    elif kind == "huge":
+        case.ham, phi0 = "burgers2d", phi0 * 1e5
+    elif kind == "tiny":
+        case.ham, phi0 = "burgers2d", phi0 * 1e-40
+    assert max(_errors(case, phi0)) <= FP64_TOL
