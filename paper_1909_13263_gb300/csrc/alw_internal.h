@@ -47,7 +47,7 @@ struct StageParams {
   double cfl, lx, ly;    // dt = cfl / (ax/lx + ay/ly)
   double alpha_fixed[2];
   double dt_value;       // LOOP_STAGE: the dt of this stage
-  int small_tiles;       // FP64 2D: 0 default tiles; 16 x 16 tiles with 4-node (1) or 2-node (2) segments
+  int shape64;           // FP64 2D: tile shape (kShape64)
   // buffers: padded arrays whose interior origin is at row GY, column GX
   const void *src0, *src1, *src2;  // stencil source (F64/F32: src0; MIXED: hi, lo, previous increment or null)
   const void *base0, *base1;       // phi^n at the node (F64/F32: base0; MIXED: hi, lo; stage>=2)
@@ -69,8 +69,22 @@ constexpr int GX = 4;   // 3 used; 4 keeps TMA box starts 16-byte aligned
 constexpr int GY = 3;
 
 // Tile shapes per variant.
+// FP64 2D tile shapes: width, height, nodes per sweep segment and the warps per SM the registers are sized for.
+// Long segments repeat less work at their ends, many small tiles spread a small grid over the SMs.
+// Microseconds per RK3 step of Example 3 (a column per shape):
+//   grid     32x16,8  16x16,8  16x8,4  16x8,2
+//   2048^2      1530     1530    1760    2190
+//    600^2       165      164     201     227
+//    400^2       111       98     111     112
+//    300^2        86       76      63      83
+//    128^2        78       76      54      38
+// so a shape serves while it gives every SM four tiles (16 x 8 with 4 nodes: three).
+struct Shape64 {
+  int tx, ty, k, warps, per_sm;
+};
+constexpr Shape64 kShape64[] = {{32, 16, 8, 20, 4}, {16, 16, 8, 20, 4}, {16, 8, 4, 16, 3}, {16, 8, 2, 16, 0}};
+constexpr int kShapes64 = sizeof(kShape64) / sizeof(kShape64[0]);
 template <int PREC> struct Tile;
-template <> struct Tile<P_F64> { static constexpr int TX = 32, TY = 16, K = 4; };
 template <> struct Tile<P_F32> { static constexpr int TX = 64, TY = 32, K = 8; };
 template <> struct Tile<P_MIXED> { static constexpr int TX = 64, TY = 32, K = 8; };
 constexpr int TX1D = 256;       // 1D tile width (one row), float variants

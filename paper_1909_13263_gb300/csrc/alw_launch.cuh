@@ -4,10 +4,10 @@
 
 namespace alw {
 
-template <int PREC, int DIM, int W, int SMALL = 0>
+template <int PREC, int DIM, int W, int SHAPE = 0>
 static int launch_one(const StageParams &p, cudaStream_t stream) {
-  using Sh = Shape<PREC, DIM, SMALL>;
-  auto kern = stage_kernel<PREC, DIM, W, SMALL>;
+  using Sh = Shape<PREC, DIM, SHAPE>;
+  auto kern = stage_kernel<PREC, DIM, W, SHAPE>;
   const size_t smem = Sh::smem_bytes();
   static bool configured = false;   // attribute is per function; setting it twice is harmless
   if (!configured) {
@@ -20,6 +20,15 @@ static int launch_one(const StageParams &p, cudaStream_t stream) {
   return (int)cudaGetLastError();
 }
 
+template <int W, int SHAPE = 0>
+static int launch_shape(const StageParams &p, cudaStream_t stream) {
+  if constexpr (SHAPE < kShapes64) {
+    if (p.shape64 == SHAPE) return launch_one<P_F64, 2, W, SHAPE>(p, stream);
+    return launch_shape<W, SHAPE + 1>(p, stream);
+  }
+  return (int)cudaErrorInvalidValue;
+}
+
 // FP64 runs here in 1D and 2D; the float variants only in 1D (2D float stages run the persistent
 // TMA kernel, so their 2D instantiations of this kernel are not built).
 template <int PREC>
@@ -27,11 +36,7 @@ static int launch_stage_impl(const StageParams &p, void *stream) {
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (p.dim == 2) {
     if constexpr (PREC == P_F64) {
-      if (p.small_tiles == 2)
-        return p.weights == W_JP ? launch_one<PREC, 2, W_JP, 2>(p, s) : launch_one<PREC, 2, W_ARCLEN, 2>(p, s);
-      if (p.small_tiles == 1)
-        return p.weights == W_JP ? launch_one<PREC, 2, W_JP, 1>(p, s) : launch_one<PREC, 2, W_ARCLEN, 1>(p, s);
-      return p.weights == W_JP ? launch_one<PREC, 2, W_JP>(p, s) : launch_one<PREC, 2, W_ARCLEN>(p, s);
+      return p.weights == W_JP ? launch_shape<W_JP>(p, s) : launch_shape<W_ARCLEN>(p, s);
     } else
       return (int)cudaErrorInvalidValue;
   }

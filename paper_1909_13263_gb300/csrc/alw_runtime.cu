@@ -114,11 +114,11 @@ void alw::dev_free(void *ptr, size_t bytes, void *stream) {
 
 int alw::tile_x(int prec, int dim) {
   if (dim == 1) return prec == P_F64 ? TX1D64 : TX1D;
-  return prec == P_F64 ? Tile<P_F64>::TX : Tile<P_F32>::TX;
+  return prec == P_F64 ? kShape64[0].tx : Tile<P_F32>::TX;
 }
 int alw::tile_y(int prec, int dim) {
   if (dim == 1) return 1;
-  return prec == P_F64 ? Tile<P_F64>::TY : Tile<P_F32>::TY;
+  return prec == P_F64 ? kShape64[0].ty : Tile<P_F32>::TY;
 }
 
 struct alw_solver {
@@ -144,7 +144,7 @@ struct alw_solver {
   cudaGraphExec_t g_adv = nullptr;
   bool has_phi = false;
   bool use2d = false;       // persistent TMA kernel (2D float variants)
-  int small_tiles = 0;      // FP64 2D: 16 x 16 tiles for grids that would not fill the GPU otherwise (1, 2)
+  int shape64 = 0;          // FP64 2D: tile shape (kShape64)
   CUtensorMap maps[6];      // tensor maps of the padded arrays (see Stage2DParams)
 
   void *alloc(size_t bytes) {
@@ -158,6 +158,20 @@ namespace {
 
 bool is_1d_ham(int k) { return k == ALW_H_ADVECT1D || k == ALW_H_BURGERS1D || k == ALW_H_NEGCOS1D ||
                                       k == ALW_H_NONCONVEX1D; }
+
+// The first FP64 tile shape that gives every SM its share of tiles (see kShape64).
+int pick_shape64(int nx, int ny) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int i = 0;
+  for (; i + 1 < kShapes64; ++i) {
+    const Shape64 &s = kShape64[i];
+    const long long tiles = (long long)((nx + s.tx - 1) / s.tx) * ((ny + s.ty - 1) / s.ty);
+    if (tiles >= (long long)s.per_sm * sms) break;
+  }
+  return i;
+}
 
 int kernel_prec(int precision) {
   return precision == ALW_PREC_FP64 ? P_F64 : precision == ALW_PREC_FP32 ? P_F32 : P_MIXED;
@@ -221,7 +235,7 @@ StageParams make_params(const alw_solver *s, int stage, int src_of, int loop_mod
   p.pitch = s->pitch;
   p.tiles_x = s->tiles_x;
   p.tiles_y = s->tiles_y;
-  p.small_tiles = s->small_tiles;
+  p.shape64 = s->shape64;
   p.dim = s->dim;
   p.bc = s->grid.bc;
   p.ham = s->ham.kind;
@@ -477,18 +491,9 @@ alw_status alw_create(const alw_grid *grid, const alw_hamiltonian *ham, const al
   s->ly = scheme->dt_mode == ALW_DT_DX53 ? std::pow(s->dy, 5.0 / 3.0) : s->dy;
   int tx = tile_x(s->prec, s->dim), ty = tile_y(s->prec, s->dim);
   if (s->dim == 2 && s->prec == P_F64) {
-    // one FP64 tile keeps an SM busy for a long time: where the default tiles would not give every SM
-    // two, 16 x 16 tiles spread the grid over four times as many CTAs
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long t = (long long)((s->nx + tx - 1) / tx) * ((s->ny + ty - 1) / ty);
-    if (sms > 0 && t < 2LL * sms) {
-      // fewer 16 x 16 tiles than SMs: 2-node segments, twice the threads per tile
-      const long long t16 = (long long)((s->nx + 15) / 16) * ((s->ny + 15) / 16);
-      s->small_tiles = t16 < sms ? 2 : 1;
-      tx = ty = 16;
-    }
+    s->shape64 = pick_shape64(s->nx, s->ny);
+    tx = kShape64[s->shape64].tx;
+    ty = kShape64[s->shape64].ty;
   }
   s->tiles_x = (s->nx + tx - 1) / tx;
   s->tiles_y = (s->ny + ty - 1) / ty;

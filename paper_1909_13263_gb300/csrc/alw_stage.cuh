@@ -10,14 +10,14 @@ namespace alw {
 // Constants of the FP64 sweeps, formed on the host (nothing for the float variants).
 template <int PREC> struct SweepArgs {};
 template <> struct SweepArgs<P_F64> {
-  Sweep64 x, y;
+  Sweep64 c[2];
 };
 template <int PREC, int W>
 static SweepArgs<PREC> sweep_args(const StageParams &p) {
   SweepArgs<PREC> a;
   if constexpr (PREC == P_F64) {
-    a.x = make_sweep64<W>(p.dx, p.eps);
-    a.y = p.dim == 2 ? make_sweep64<W>(p.dy, p.eps) : a.x;
+    a.c[0] = make_sweep64<W>(p.dx, p.eps);
+    a.c[1] = p.dim == 2 ? make_sweep64<W>(p.dy, p.eps) : a.c[0];
   }
   return a;
 }
@@ -109,46 +109,29 @@ template <> struct Types<P_F64> { using S = double; using C = double; };
 template <> struct Types<P_F32> { using S = float; using C = float; };
 template <> struct Types<P_MIXED> { using S = float; using C = float; };
 
-// SMALL (FP64 2D grids too small to fill the GPU with the default tiles): 16 x 16 tiles with 4-node
-// sweep segments (SMALL = 1), or 2-node segments (SMALL = 2: twice the threads per tile, for grids
-// whose 16 x 16 tiles are fewer than the SMs).
-template <int PREC, int DIM, int SMALL = 0> struct Shape {
-  static constexpr int TX = (DIM == 2) ? (SMALL ? 16 : Tile<PREC>::TX) : (PREC == P_F64 ? TX1D64 : TX1D);
-  static constexpr int TY = (DIM == 2) ? (SMALL ? 16 : Tile<PREC>::TY) : 1;
-  static constexpr int K = (DIM == 2) ? (SMALL == 2 ? 2 : SMALL == 1 ? 4 : Tile<PREC>::K) : (PREC == P_F64 ? 1 : K1D);
-  static constexpr int NT = (TX / K) * TY;          // threads per CTA
-  static constexpr int MINB = (PREC == P_F64 && DIM == 2) ? 512 / NT : 1;   // FP64: 16 warps per SM
+// SHAPE: tile shape of the FP64 2D grids.  In 2D half of the threads sweep rows and half columns.
+template <int PREC, int DIM, int SHAPE = 0> struct Shape {
+  static constexpr int TX = (DIM == 2) ? kShape64[SHAPE].tx : (PREC == P_F64 ? TX1D64 : TX1D);
+  static constexpr int TY = (DIM == 2) ? kShape64[SHAPE].ty : 1;
+  static constexpr int K = (DIM == 2) ? kShape64[SHAPE].k : (PREC == P_F64 ? 1 : K1D);
+  static constexpr int NSEG = (TX / K) * TY;        // segments per direction
+  static constexpr int NT = NSEG * DIM;             // threads per CTA
+  static constexpr int MINB = (PREC == P_F64 && DIM == 2) ? kShape64[SHAPE].warps * 32 / NT : 1;
   static constexpr int SW = TX + 8;                 // smem row: GX halo on each side
   static constexpr int SH = (DIM == 2) ? TY + 6 : 1;
   static constexpr int NARR = (PREC == P_MIXED) ? 3 : 1;
   static constexpr size_t smem_bytes() {
     return (size_t)NARR * SH * SW * sizeof(typename Types<PREC>::S) +
-           (DIM == 2 ? (size_t)TY * TX * 2 * sizeof(typename Types<PREC>::C) : 0);
+           (PREC == P_F64 ? (size_t)DIM * TY * TX * 2 * (sizeof(double) + sizeof(short)) : 0);  // derivatives, list
   }
 };
 
-// FP64: one-sided derivatives of K consecutive nodes from the cells a, a + step, ... (a = first node - 3) with
-// the weights in float pairs; nv nodes of the segment count.  False when the segment does not qualify (and
-// for the float variants).
-template <int PREC, int K, int W, class S, class C>
-__device__ __forceinline__ bool sweep_pairs(const S *a, int step, const SweepArgs<PREC> &sw, bool along_y, int nv,
-                                            C (&dm)[K], C (&dp)[K]) {
-  if constexpr (PREC == P_F64) {
-    return sweep64<K, W>([&](int m) { return a[m * step]; }, along_y ? sw.y : sw.x, nv, [&](int q, double x, double y) {
-      dm[q] = x;
-      dp[q] = y;
-    });
-  } else {
-    return false;
-  }
-}
-
-template <int PREC, int DIM, int WEIGHTS, int SMALL>
-__global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT, Shape<PREC, DIM, SMALL>::MINB)
+template <int PREC, int DIM, int WEIGHTS, int SHAPE>
+__global__ void __launch_bounds__(Shape<PREC, DIM, SHAPE>::NT, Shape<PREC, DIM, SHAPE>::MINB)
     stage_kernel(const StageParams p, const SweepArgs<PREC> sw) {
   using S = typename Types<PREC>::S;
   using C = typename Types<PREC>::C;
-  using Sh = Shape<PREC, DIM, SMALL>;
+  using Sh = Shape<PREC, DIM, SHAPE>;
   constexpr int TX = Sh::TX, TY = Sh::TY, K = Sh::K, NT = Sh::NT, SW = Sh::SW, SH = Sh::SH;
 
   DevState *st = p.state;
@@ -161,7 +144,7 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT, Shape<PREC, DIM, 
   S *s_c = s_b + SH * SW;                               // previous stage's increment (MIXED)
   C *s_u = reinterpret_cast<C *>(smem_raw + (size_t)Sh::NARR * SH * SW * sizeof(S));
   __shared__ double s_red[2][NT / 32];
-  __shared__ int s_last;
+  __shared__ int s_last, s_nrare;
 
   const int tid = threadIdx.x;
   const int tx0 = blockIdx.x * TX, ty0 = blockIdx.y * TY;
@@ -202,6 +185,7 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT, Shape<PREC, DIM, 
     fay = C(bits_to_double(st->alpha_bits[p.read_slot][1]));
   }
 
+  if (tid == 0) s_nrare = 0;
   // ---- load the tile and its halo (row 0 of smem = interior row ty0-3, col 0 = interior col tx0-4)
   const S *ga = reinterpret_cast<const S *>(PREC == P_MIXED ? p.mix_hi[cur] : p.src0);
   const S *gb = reinterpret_cast<const S *>(PREC == P_MIXED ? p.mix_lo[cur] : nullptr);
@@ -297,53 +281,61 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SMALL>::NT, Shape<PREC, DIM, 
     }
   };
 
-  // nodes of a K-node segment that lie inside the grid
-  auto valid = [&](int left, bool inside) { return !inside || left <= 0 ? -9 : (left < K ? left : K); };
-
-  // ---- phase X: each thread sweeps K consecutive nodes of one row
-  {
-    constexpr int SEGS = TX / K;
-    const int r = tid / SEGS, seg = tid - r * SEGS;
-    const int srow = (DIM == 2) ? r + 3 : 0;
-    const int base_i = srow * SW + seg * K + 1;     // smem index of node x = seg*K - 3
-    C dm[K], dp[K];
-    const int nv = valid(p.nx - tx0 - seg * K, DIM == 1 || ty0 + r < p.ny);
-    if (!sweep_pairs<PREC, K, WEIGHTS>(s_a + base_i, 1, sw, false, nv, dm, dp)) {
-      C v[K + 5];
-#pragma unroll
-      for (int m = 0; m < K + 5; ++m) v[m] = diff(base_i + m, base_i + m + 1, rdx);
-      weno_sweep<C, K, WEIGHTS>(v, rdx, dx, eps, dm, dp);
-    }
-    if (DIM == 2) {
-#pragma unroll
-      for (int q = 0; q < K; ++q) {
-        s_u[2 * (r * TX + seg * K + q)] = dm[q];
-        s_u[2 * (r * TX + seg * K + q) + 1] = dp[q];
+  if constexpr (PREC == P_F64) {
+    // each thread sweeps K consecutive nodes of one row or one column, one code for both (see
+    // alw_sweep64.cuh); the results go through shared memory, so that the sweep's loop holds nothing of what
+    // finishing a node needs (registers)
+    double2 *su = reinterpret_cast<double2 *>(s_u), *sv = su + (DIM - 1) * TY * TX;
+    unsigned short *s_rare = reinterpret_cast<unsigned short *>(su + DIM * TY * TX);
+    {
+      constexpr int SEGS = TX / K;
+      const int dir = (DIM == 2 && tid >= Sh::NSEG) ? 1 : 0, seg = tid - dir * Sh::NSEG;
+      const int x = dir == 0 ? (seg % SEGS) * K : seg % TX, y = dir == 0 ? seg / SEGS : (seg / TX) * K;
+      const S *a = s_a + (DIM == 2 ? y + (dir == 0 ? 3 : 0) : 0) * SW + x + (dir == 0 ? 1 : 4);
+      const int step = dir == 0 ? 1 : SW, ostep = dir == 0 ? 1 : TX, node0 = y * TX + x;
+      // nodes of the segment that lie inside the grid
+      const int left = dir == 0 ? p.nx - tx0 - x : p.ny - ty0 - y;
+      const bool inside = dir == 0 ? (DIM == 1 || ty0 + y < p.ny) : tx0 + x < p.nx;
+      double2 *o = (dir == 0 ? su : sv) + node0;
+      unsigned rare = sweep64<WEIGHTS>(a, step, sw.c[dir], !inside || left <= 0 ? -1 : (left < K ? left : K),
+                                       [&](int q, double dm, double dp) { o[q * ostep] = make_double2(dm, dp); });
+      // nodes that did not qualify: both sides of each into the CTA's list
+      while (rare) {
+        const int q = __ffs(rare) - 1;
+        rare &= rare - 1;
+        const int at = atomicAdd(&s_nrare, 2);
+        s_rare[at] = (unsigned short)(((dir * TY * TX + node0 + q * ostep) << 1));
+        s_rare[at + 1] = (unsigned short)(s_rare[at] | 1);
       }
-    } else {
-#pragma unroll
-      for (int q = 0; q < K; ++q) finish_node(seg * K + q, 0, dm[q], dp[q], C(0), C(0));
     }
-  }
-  if (DIM == 2) {
     __syncthreads();
-    // ---- phase Y: each thread sweeps K consecutive nodes of one column
-    const int x = tid % TX, seg = tid / TX;
-    const int col = x + 4;
-    const C dy = C(p.dy), rdy = C(p.rdy);
-    C vm[K], vp[K];
-    const int nv = valid(p.ny - ty0 - seg * K, tx0 + x < p.nx);
-    if (!sweep_pairs<PREC, K, WEIGHTS>(s_a + seg * K * SW + col, SW, sw, true, nv, vm, vp)) {
-      C v[K + 5];
-#pragma unroll
-      for (int m = 0; m < K + 5; ++m) v[m] = diff((seg * K + m) * SW + col, (seg * K + m + 1) * SW + col, rdy);
-      weno_sweep<C, K, WEIGHTS>(v, rdy, dy, eps, vm, vp);
+    if (s_nrare > 0) {
+      // ... which all threads share: the kinks of a tile touch few threads' segments
+      for (int i = tid; i < s_nrare; i += NT) {
+        const int e = s_rare[i] >> 1, dir = e / (TY * TX), n = e % (TY * TX), x = n % TX, y = n / TX;
+        const int step = dir == 0 ? 1 : SW;
+        const S *a = s_a + (DIM == 2 ? y + (dir == 0 ? 3 : 0) : 0) * SW + x + (dir == 0 ? 1 : 4);
+        double *o = reinterpret_cast<double *>((dir == 0 ? su : sv) + n);
+        if (s_rare[i] & 1) o[1] = -minus64_rare<WEIGHTS>(a + 6 * step, -step, sw.c[dir]);
+        else o[0] = minus64_rare<WEIGHTS>(a, step, sw.c[dir]);
+      }
+      __syncthreads();
     }
-#pragma unroll
-    for (int q = 0; q < K; ++q) {
-      const int y = seg * K + q;
-      finish_node(x, y, s_u[2 * (y * TX + x)], s_u[2 * (y * TX + x) + 1], vm[q], vp[q]);
+#pragma unroll 1
+    for (int n = tid; n < TX * TY; n += NT) {
+      const double2 u = su[n], v = DIM == 2 ? sv[n] : make_double2(0.0, 0.0);
+      finish_node(n % TX, n / TX, u.x, u.y, v.x, v.y);
     }
+  } else {
+    static_assert(PREC == P_F64 || DIM == 1, "2D float stages run the persistent kernel");
+    const int base_i = tid * K + 1;     // smem index of the segment's first node - 3
+    C v[K + 5];
+#pragma unroll
+    for (int m = 0; m < K + 5; ++m) v[m] = diff(base_i + m, base_i + m + 1, rdx);
+    C dm[K], dp[K];
+    weno_sweep<C, K, WEIGHTS>(v, rdx, dx, eps, dm, dp);
+#pragma unroll
+    for (int q = 0; q < K; ++q) finish_node(tid * K + q, 0, dm[q], dp[q], C(0), C(0));
   }
 
   // ---- grid maximum of alpha: warp shuffle, then one atomicMax per CTA
