@@ -101,6 +101,10 @@ void set_last_error(const char *msg);
 int launch_stage_f64(const StageParams &p, void *stream);
 int launch_stage_f32(const StageParams &p, void *stream);
 int launch_stage_mixed(const StageParams &p, void *stream);
+// nsteps RK3 steps (fewer when t reaches t_final) of a 1D FP64 grid of at most kLine64Max nodes in one launch;
+// p: the parameters of stage 3 (out0 = phi^n).  Not for the exact alpha modes.
+constexpr int kLine64Max = 1024;
+int launch_line64(const StageParams &p, int nsteps, void *stream);
 int launch_ghosts(const GhostParams &g, void *stream);
 int launch_mixed_split(const double *src, void *hi, void *lo, int nx, int ny, int pitch, int dim, void *stream);
 int launch_mixed_join(const void *hi, const void *lo, const void *delta, double *dst, int nx, int ny,

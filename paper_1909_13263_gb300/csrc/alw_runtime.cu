@@ -143,6 +143,7 @@ struct alw_solver {
   int g_step_n = 0;
   cudaGraphExec_t g_adv = nullptr;
   bool has_phi = false;
+  bool line64 = false;      // 1D FP64 grid that fits one cluster: many steps per launch
   bool use2d = false;       // persistent TMA kernel (2D float variants)
   int shape64 = 0;          // FP64 2D: tile shape (kShape64)
   CUtensorMap maps[6];      // tensor maps of the padded arrays (see Stage2DParams)
@@ -315,6 +316,8 @@ GhostParams ghost_params(const alw_solver *s, int after_stage) {
   }
   return g;
 }
+
+constexpr int kLineSteps = 512;  // RK3 steps per launch of the 1D FP64 cluster kernel (a few ms)
 
 // Enqueue one RK3 step (with the reduction passes and ghost fills the mode needs).
 alw_status enqueue_step(alw_solver *s, int loop_mode) {
@@ -501,6 +504,7 @@ alw_status alw_create(const alw_grid *grid, const alw_hamiltonian *ham, const al
   s->rows = s->dim == 2 ? s->tiles_y * ty + 2 * GY : 1;
   s->elem = s->prec == P_F64 ? 8 : 4;
   s->use2d = s->dim == 2 && s->prec != P_F64;
+  s->line64 = s->dim == 1 && s->prec == P_F64 && s->nx <= kLine64Max && !exact_mode(s->alpha_mode);
   s->arr_bytes = (size_t)s->pitch * s->rows * s->elem;
 
   auto cleanup = [&](alw_status st) {
@@ -608,7 +612,9 @@ alw_status alw_step_to(alw_solver *s, double t_final, int64_t *steps_out) {
   alw_status st = check_solver(s);
   if (st) return st;
   if (!std::isfinite(t_final)) return fail(ALW_EINVAL, "t_final must be finite");
-  if (!s->g_step) {
+  if (s->line64) {
+    s->g_step_n = kLineSteps;
+  } else if (!s->g_step) {
     s->g_step_n = (s->nx * (long long)s->ny >= (1 << 22)) ? 4 : 16;
     st = build_graph(s, LOOP_STEP_TO, s->g_step_n, &s->g_step);
     if (st) return st;
@@ -627,7 +633,10 @@ alw_status alw_step_to(alw_solver *s, double t_final, int64_t *steps_out) {
     if (!(s->h_st->t < t_final)) break;
     const double t_prev = s->h_st->t;
     const int64_t steps_prev = s->h_st->steps;
-    for (int r = 0; r < replays; ++r) ALW_CUDA(cudaGraphLaunch(s->g_step, s->stream));
+    for (int r = 0; r < replays; ++r) {
+      if (s->line64) ALW_LAUNCH(launch_line64(make_params(s, 3, 3, LOOP_STEP_TO), kLineSteps, s->stream));
+      else ALW_CUDA(cudaGraphLaunch(s->g_step, s->stream));
+    }
     st = read_state(s);
     if (st) return st;
     if (freeze > 0 && ++reads >= freeze) {
@@ -659,6 +668,13 @@ alw_status alw_advance(alw_solver *s, int64_t nsteps) {
   alw_status st = check_solver(s);
   if (st) return st;
   if (nsteps < 0) return fail(ALW_EINVAL, "nsteps < 0");
+  if (s->line64) {
+    for (int64_t i = 0; i < nsteps; i += kLineSteps) {
+      const int k = (int)(nsteps - i < kLineSteps ? nsteps - i : kLineSteps);
+      ALW_LAUNCH(launch_line64(make_params(s, 3, 3, LOOP_ADVANCE), k, s->stream));
+    }
+    return ALW_OK;
+  }
   if (!s->g_adv) {
     st = build_graph(s, LOOP_ADVANCE, 1, &s->g_adv);
     if (st) return st;

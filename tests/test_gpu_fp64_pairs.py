@@ -77,3 +77,60 @@ def test_mixed_segments_match_oracle(kind, weights):
     elif kind == "tiny":
         case.ham, phi0 = "burgers2d", phi0 * 1e-40
     assert max(_errors(case, phi0)) <= FP64_TOL
+
+
+# 1D grids that run whole steps in one launch (up to 1024 nodes): edges of the shares of 1, 2, 4 and 8 CTAs
+@pytest.mark.parametrize("nx", [2, 5, 64, 65, 128, 129, 257, 513, 1024, 1025])
+@pytest.mark.parametrize("kw", [dict(bc="periodic"), dict(bc="linextrap", alpha_mode="global_lagged"),
+                                dict(bc="periodic", weights="jp", alpha_mode="fixed", alpha_fixed=(5.0, 0.0)),
+                                dict(bc="linextrap", dt_mode="dx53")], ids=lambda k: "-".join(map(str, k.values())))
+def test_line_solve_matches_oracle(nx, kw):
+    case = Case(1, nx, 1, "burgers1d", **{"alpha_mode": "local_lagged", **kw})
+    x, _ = inputs.axis(nx, -1.0, 1.0, case.bc)
+    phi0 = -np.cos(np.pi * x + 0.3) + 0.2 * np.abs(x)
+    a, _ = oracle.alpha_of(case.cfg(), phi0)
+    alpha = case.alpha_fixed[0] if case.alpha_mode == "fixed" else a[0]
+    tf = 7.5 * 0.6 * (case.dx ** (5.0 / 3.0) if case.dt_mode == "dx53" else case.dx) / alpha
+    ref, steps_ref, t_ref, _, st = oracle.solve(case.cfg(), phi0, tf)
+    assert st == 0
+    with case.solver() as s:
+        s.set_phi0(phi0)
+        n = s.step_to(0.4 * tf)
+        mid, state = s.get_phi(), s.get_state()
+        n += s.step_to(tf)
+        whole, end = s.get_phi(), s.get_state()
+        # resumed from the state in between: the same bits
+        s.set_state(state, mid)
+        s.step_to(tf)
+        assert np.array_equal(s.get_phi(), whole)
+        # the same number of steps without clipping, then one per-stage step on top of it
+        s.set_phi0(phi0)
+        s.advance(3)
+        s.advance(2)
+        five = s.get_phi()
+        s.set_phi0(phi0)
+        s.advance(5)
+        assert np.array_equal(s.get_phi(), five)
+        assert s.get_state().steps == 5
+    assert end.t == t_ref == tf
+    # one extra step at most where the run was stopped in between
+    assert steps_ref <= n <= steps_ref + 1
+    with case.solver() as s:
+        s.set_phi0(phi0)
+        assert s.step_to(tf) == steps_ref
+        assert rel_err(s.get_phi(), ref) <= FP64_TOL
+
+
+def test_line_solve_reports_nonfinite():
+    case = Case(1, 200, 1, "burgers1d", alpha_mode="local_lagged")
+    phi0 = case.field(seed=2, kind="smooth")
+    with case.solver() as s:
+        s.set_phi0(phi0)
+        s.advance(1)
+        bad = s.get_phi()
+        bad[77] = np.nan
+        s.set_state(s.get_state(), bad)
+        with pytest.raises(native.AlwError) as e:
+            s.step_to(1.0)
+        assert e.value.status == native.ENONFINITE
+        assert s.get_state().steps == 1
