@@ -209,9 +209,6 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
   constexpr int SW = G::SW, SH = G::SH, ARR = G::ARR;
   constexpr int DXW = G::DXW, DXP = G::DXP, SUP = G::SUP, CG = G::CG;
   constexpr int NARR = (PREC == P_MIXED) ? 3 : 2;
-  // arc length with the increment form (MIXED): try the short-interval sweep first (FP32 stores phi
-  // itself, whose rounding makes second differences rough at fine grids, so it never qualifies there)
-  constexpr bool SHORT = (W == W_ARCLEN && PREC == P_MIXED);
   const StageParams &p = prm.p;
   const bool batch = prm.insts != nullptr;
   if (!batch) {
@@ -412,9 +409,8 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     // finish loop)
     const float *X = (PREC == P_MIXED && prm.map_c >= 0) ? C : B;
 
-    // ---- 1. x differences in the units of the sweep (arc length: Delta^+ phi / dx^2; Jiang-Peng:
-    // Delta^+ phi / dx), rows by warp, columns by lane (no division, conflict-free)
-    const float rdx2 = (W == W_ARCLEN) ? d.rdx * d.rdx : d.rdx;
+    // ---- 1. x differences Delta^+ phi / dx, rows by warp, columns by lane (no division, conflict-free)
+    const float rdx1 = d.rdx;
     {
       auto cell_diff = [&](int i0, int i1) -> float {
         if (PREC == P_MIXED) return (A[i1] - A[i0]) + (X[i1] - X[i0]);
@@ -427,13 +423,13 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
 #pragma unroll
         for (int c = lane; c < TX; c += 32) {
           const int i0 = (r + 3) * SW + c + 1;
-          dX[r * DXP + c] = cell_diff(i0, i0 + 1) * rdx2;
+          dX[r * DXP + c] = cell_diff(i0, i0 + 1) * rdx1;
         }
       }
       for (int j = tid; j < TY * (DXW - TX); j += NT) {
         const int r = j / (DXW - TX), c = TX + j % (DXW - TX);
         const int i0 = (r + 3) * SW + c + 1;
-        dX[r * DXP + c] = cell_diff(i0, i0 + 1) * rdx2;
+        dX[r * DXP + c] = cell_diff(i0, i0 + 1) * rdx1;
       }
     }
     if (__syncthreads_or(!ok)) {
@@ -460,7 +456,7 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
       // differences of the differences pass (in the same units); u_at is called for m = 0, 1, 2, ... in
       // order, so each position loads one new row and reuses the previous one
       const int iy = (K * segY) * SW + colY + 4;
-      const float rdy2 = (W == W_ARCLEN) ? d.rdy * d.rdy : d.rdy;
+      const float rdy1 = d.rdy;
       auto make_vat = [&]() {
         float pa = A[iy], px = 0.0f;
         if (PREC == P_MIXED) px = X[iy];
@@ -477,7 +473,7 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
             dy = a1 - pa;
             pa = a1;
           }
-          return make_float2(vx[m], dy * rdy2);
+          return make_float2(vx[m], dy * rdy1);
         };
       };
       auto emit = [&](int q, float2 dm, float2 dp) {
@@ -490,17 +486,31 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
       sc.h2 = make_float2(0.5f * d.dx, 0.5f * d.dy);
       sc.h3 = make_float2(d.dx * (1.0f / 3.0f), d.dy * (1.0f / 3.0f));
       sc.mh6 = make_float2(d.dx * (-1.0f / 6.0f), d.dy * (-1.0f / 6.0f));
-      // arc length, MIXED: every warp sweeps with the short-interval form first and sweeps again in
-      // full when some segment of the warp does not qualify (that form then replaces all its
-      // results).  Which form produced a node's values thus depends only on the data of the warp's
-      // segments, whose position on the grid is fixed by the tile width -- not on the order in
-      // which tiles or instances are processed, nor on history: a single solve, a batch, a server
-      // round and a resumed checkpoint (all with 64-wide tiles) choose alike.
-      bool full = true;
-      if (SHORT) full = !sweep_stream_short<K, float2>(make_vat(), sc, emit);
-      if (full) {
-        if constexpr (W == W_ARCLEN) sweep_stream<K, float2>(make_vat(), sc, emit);
-        else sweep_stream_jp<K, float2>(make_vat(), make_float2(eps, eps), emit);
+      // arc length: every warp sweeps with the near-linear form first and sweeps again in full when some
+      // segment of the warp does not qualify (that form then replaces all its results).  Which form
+      // produced a node's values thus depends only on the data of the warp's segments, whose position on
+      // the grid is fixed by the tile width -- not on the order in which tiles or instances are processed,
+      // nor on history: a single solve, a batch, a server round and a resumed checkpoint (all with
+      // 64-wide tiles) choose alike.
+      if constexpr (W == W_ARCLEN) {
+        const float2 rd = make_float2(d.rdx, d.rdy);
+        // FP32 stores phi itself: its rounding over dx is what the derivatives carry anyway
+        float2 size = make_float2(0.0f, 0.0f);
+        if (PREC == P_F32) {
+          const int ix = (lane + 3) * SW + K * warp + 4;
+          size = make_float2(fmaxf(fabsf(A[ix]), fabsf(A[ix + K - 1])) * d.rdx,
+                             fmaxf(fabsf(A[iy + 3 * SW]), fabsf(A[iy + (K + 2) * SW])) * d.rdy);
+        }
+        // segments of rows or columns beyond the grid (ragged tiles) do not count
+        if (ty0 + lane >= ny || tx0 + K * warp >= nx) size.x = INFINITY;
+        if (tx0 + colY >= nx || ty0 + K * segY >= ny) size.y = INFINITY;
+        if (!sweep_stream_near<K, float2>(make_vat(), rd, make_float2(fmaf(d.dx, d.dx, eps), fmaf(d.dy, d.dy, eps)),
+                                          size, emit)) {
+          auto v_at = make_vat();
+          sweep_stream<K, float2>([&](int m) { return vmul(v_at(m), rd); }, sc, emit);
+        }
+      } else {
+        sweep_stream_jp<K, float2>(make_vat(), make_float2(eps, eps), emit);
       }
     }
     __syncthreads();

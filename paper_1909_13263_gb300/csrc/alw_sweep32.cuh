@@ -30,20 +30,21 @@
 // multiply; dx enters once, in the constants dx/2, dx/3, -dx/6 of the central parts and of T_a/3, T_b/2.
 // The Jiang-Peng sweep needs no D2 and keeps v.
 //
-// Short intervals.  The interval mean G takes the trapezoid value (s_a + s_b) / 2 whenever the
-// interval [a, b] is short against its end values (|b - a| <= (s_a + s_b) / 64, s = sqrt(1 + u^2)).
-// On smooth data at fine grids every interval of a segment is that short (its width is a third
-// difference of phi over dx^2, about phi_xxx dx), and then F, its logarithm and the interval
-// reciprocals are never used.  sweep_stream_short computes only what the trapezoid branch needs
-// and reports whether the segment qualifies: every width W_m of the segment at most
-// kShortH (which implies the trapezoid branch for all three interval kinds, because D2_{m+1} - D2_m
-// is such a width and R_m - D2_m and D2_m - L_m equal one up to the rounding of R or L -- below 1e-4
-// while |D2| <= kShortD2, against the margin 1/32 - kShortH -- and s >= 1), |D2| at the segment
-// start at most kShortD2 and eps4 at most kShortEps4 (together
-// these keep every weight denominator below 1e29, so the overflow branch of group_corr_v is not
-// needed).  When the segment qualifies, both sweeps evaluate the same formulas on the same branches;
-// their results agree to rounding (the compiler may select instructions for the two code paths
-// differently), and the stage kernel decides between them from the segment's own data only.
+// Near-linear segments.  On data the grid resolves the weights differ from the linear ones by small amounts, and
+// what they contribute is that difference times third differences.  With all q's of a stencil within a factor
+// 1 + eta of each other, e = eps + (dx G)^2, y = dx times the middle of the stencil's central interval (so that
+// G^2 = 1 + (y/dx)^2 to the order kept) and (a, b) the stencil's two third differences T, the indicators'
+// differences are -a y and -b y and the deviations from the linear scheme
+//   phi^- = lin^- - k (6 a^2 - 3 a b + 7 b^2)/100,   phi^+ = lin^+ + k (7 a^2 - 3 a b + 6 b^2)/100,  k = y/(y^2 + dx^2 + eps),
+//   lin^-+ = (v_2 + v_3)/2 -+ ... = (v_2 + v_3)/2 + W_1/30 - 3 W_2/20 - W_3/20  ("+": mirrored, from W_4),
+// one reciprocal and no square root per stencil for both sides.  sweep_stream_near evaluates this and bounds what
+// it leaves out: in units of D2 = dx^2-scaled differences (T, W the segment's largest) second-order terms
+// of the weights (0.04 T^3), of the indicators (0.01 T^3) and the interval widths' share of them
+// (0.01 T^2 W + 0.0025 T^2 W^2).  The segment qualifies when that is at most 2^-25 of its largest difference
+// (half a unit of the derivatives' own rounding), or, for a phi stored in float, 2^-25 of |phi| / dx (the
+// rounding of phi itself).  |y|/(y^2 + dx^2) <= 1/(2 dx), whence the bounds hold for any y.  A warp whose
+// segments do not all qualify sweeps them again with sweep_stream; the choice depends on the segments' own
+// data only.
 #pragma once
 #include <type_traits>
 
@@ -57,9 +58,7 @@
 
 namespace alw {
 
-constexpr float kShortH = 0.03f;      // largest width D2_{m+1} - D2_m of a short segment
-constexpr float kShortD2 = 400.0f;    // largest |D2| at the start of a short segment
-constexpr float kShortEps4 = 1.0e6f;  // largest 4 eps / dx^2 of a short segment
+constexpr float kNearTol = 1.0f / 33554432.0f;  // 2^-25
 
 // ---- lane-wise operations on float and float2 ------------------------------------------
 // Every add, subtract and multiply is rounded as written: the packed forms are PTX instructions
@@ -259,27 +258,6 @@ __device__ __forceinline__ void group_corr_v(V g0, V g1, V g2, V ta_m, V tb_m, V
   if (PLUS) side(p01, p12, ta_p, tb_p, false, g2, g1, g0, num_p, r_p);
 }
 
-// Every lane of v holds a width at most kShortH (NaN fails).
-template <class V>
-__device__ __forceinline__ bool short_width(V h) {
-  using LN = Lanes<V>;
-  bool ok = true;
-#pragma unroll
-  for (int i = 0; i < LN::n; ++i) ok &= fabsf(LN::get(h, i)) <= kShortH;
-  return ok;
-}
-
-// The size conditions of a short segment on |D2| at its start and on eps4 (NaN fails).
-template <class V>
-__device__ __forceinline__ bool short_sizes(V d2, V eps4) {
-  using LN = Lanes<V>;
-  bool ok = true;
-#pragma unroll
-  for (int i = 0; i < LN::n; ++i)
-    ok &= (fabsf(LN::get(d2, i)) <= kShortD2) & (LN::get(eps4, i) <= kShortEps4);
-  return ok;
-}
-
 // The extrapolated interval ends R_m = 2 D2_m - D2_{m-1} and L_m = 2 D2_m - D2_{m+1}, formed as
 // D2_m plus or minus the neighbouring width W (the quantity the short-interval test inspects; one
 // operation each).
@@ -424,71 +402,87 @@ __device__ __forceinline__ void sweep_stream_jp(LoadV v_at, V eps, Emit emit) {
   }
 }
 
-// Arc-length sweep of segments on which every interval takes the trapezoid branch (see the header
-// comment): the square roots s = sqrt(1 + u^2) of the interval ends, the trapezoid values and the
-// weights, with the operations of sweep_stream on those branches.  Called by all 32 threads of a
-// warp; returns, uniformly across the warp, whether every segment of the warp (both lanes of all
-// threads) met the conditions (checked after the prologue, where a failing warp stops at once,
-// and after the last node).  When it returns false the emitted values, if any, are not to be
-// used and the caller sweeps the warp's segments again with sweep_stream.
+// Near-linear arc-length sweep (see the header comment), in units of the first differences: v_at(m) returns
+// v = Delta^+ phi / dx at position i0 - 3 + m; rdx per lane; e1 = dx^2 + eps; size: what errors are measured
+// against besides the segment's |v| (0, or |phi| / dx).  Called by all 32 threads of a warp; returns, uniformly
+// across the warp, whether every segment of the warp (both lanes of all threads) qualified (checked after
+// the first stencil, where a failing warp stops at once, and after the last).  When it returns false
+// the emitted values, if any, are not to be used and the caller sweeps the warp's segments with sweep_stream.
 template <int K, class V, class LoadV, class Emit>
-__device__ __forceinline__ bool sweep_stream_short(LoadV u_at, const SweepConsts<V> &c, Emit emit) {
-  Window<K + 5, V> w;
-  V S[K + 6];                                // S_m = sqrt(1 + D2_m^2)
-  V qX[K + 6], qY[K + 6], qZ[K + 6];
-  bool ok = true;
-
-  auto sq = [&](V u) { return s_eval_v(u); };   // FValV::s of f_eval_v
-  auto qv = [&](V sa, V sb) {                // q of q_interval_v on its trapezoid branch
-    const V ss = vadd(sa, sb);
-    const V e = vfma(ss, ss, c.eps4);
-    return vmul(e, e);
-  };
+__device__ __forceinline__ bool sweep_stream_near(LoadV v_at, V rdx, V e1, V size, Emit emit) {
+  using LN = Lanes<V>;
+  V v[K + 5], D[K + 5], W[K + 5], T[K + 5], TT[K + 5];   // TT_m = T_m^2
+  V tm = vsplat(0.0f, e1);                               // largest |T|
+  auto c = [&](float x) { return vsplat(x, e1); };
   auto pos = [&](int m) {
-    w.pos(m, c);
-    if (m >= 2) ok &= short_width(w.W[m - 1]);
+    if (m >= 1) D[m] = vsub(v[m], v[m - 1]);
+    if (m >= 2) W[m - 1] = vsub(D[m], D[m - 1]);
+    if (m >= 3) {
+      T[m - 1] = vsub(W[m - 1], W[m - 2]);
+      TT[m - 1] = vmul(T[m - 1], T[m - 1]);
+#pragma unroll
+      for (int i = 0; i < LN::n; ++i) LN::at(tm, i) = fmaxf(LN::get(tm, i), fabsf(LN::get(T[m - 1], i)));
+    }
   };
-  auto al_qX = [&](int m) { qX[m] = qv(S[m], sq(r_end(w.D2[m], w.W[m - 1]))); };
-  auto al_qY = [&](int m) { qY[m] = qv(S[m], S[m + 1]); };
-  auto al_qZ = [&](int m) { qZ[m] = qv(sq(l_end(w.D2[m], w.W[m])), S[m]); };
-  // the denominators stay in range on short segments: no check
-  auto stencil = [&](int j, auto minus_c, auto plus_c, V &nm, V &rm, V &np, V &rp) {
-    constexpr bool MI = decltype(minus_c)::value, PL = decltype(plus_c)::value;
-    group_corr_v<false, MI, PL>(qX[j + 2], qY[j + 2], qZ[j + 3], w.Ta[j + 2], w.Tb[j + 3], w.Ta[j + 3],
-                                w.Tb[j + 2], nm, rm, np, rp);
+  // stencil j: -k of the "-" side and both quadratic forms
+  auto stencil = [&](int j, V &nk, V &qm, V &qp) {
+    const V y = vfma(c(0.5f), W[j + 2], D[j + 2]);
+    const V e = vfma(y, y, e1);
+    V r;
+#pragma unroll
+    for (int i = 0; i < LN::n; ++i) LN::at(r, i) = sfu_rcp(-LN::get(e, i));
+    nk = vmul(y, r);
+    const V ab = vmul(T[j + 2], T[j + 3]);
+    qm = vfma(c(0.06f), TT[j + 2], vfma(c(0.07f), TT[j + 3], vmul(c(-0.03f), ab)));
+    qp = vfma(c(-0.07f), TT[j + 2], vfma(c(-0.06f), TT[j + 3], vmul(c(0.03f), ab)));
+  };
+  // what the segment's largest T and W leave out, against its size
+  auto fits = [&](V vm) {
+    const V t = vmul(tm, rdx);
+    V w;                                                  // |W| <= |W_1| + 12 |T|
+#pragma unroll
+    for (int i = 0; i < LN::n; ++i) LN::at(w, i) = fabsf(LN::get(W[1], i)) * LN::get(rdx, i);
+    w = vfma(c(12.0f), t, w);
+    const V f = vfma(w, vfma(c(0.0025f), w, c(0.01f)), vmul(c(0.05f), t));
+    const V lhs = vmul(vmul(tm, t), f);                   // T^2 / dx (...) in units of v
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < LN::n; ++i) {
+      const float ref = fmaxf(LN::get(vm, i), LN::get(size, i));
+      ok &= LN::get(lhs, i) <= kNearTol * ref;
+    }
+    return __all_sync(0xffffffffu, ok);
+  };
+  auto vmax = [&](V a, V b) {
+    V r;
+#pragma unroll
+    for (int i = 0; i < LN::n; ++i) LN::at(r, i) = fmaxf(fabsf(LN::get(a, i)), fabsf(LN::get(b, i)));
+    return r;
   };
 
 #pragma unroll
-  for (int m = 0; m <= 5; ++m) w.u[m] = u_at(m);
-#pragma unroll
-  for (int m = 1; m <= 5; ++m) pos(m);
-#pragma unroll
-  for (int m = 2; m <= 4; ++m) S[m] = sq(w.D2[m]);
-  al_qX(2); al_qY(2); al_qZ(3);
-  al_qX(3); al_qY(3); al_qZ(4);
-  ok &= short_sizes(w.D2[2], c.eps4);
-  if (!__all_sync(0xffffffffu, ok)) return false;
-
-  V nm, rm, dummy0, dummy1;
-  stencil(0, std::true_type{}, std::false_type{}, nm, rm, dummy0, dummy1);
+  for (int m = 0; m <= 4; ++m) {
+    v[m] = v_at(m);
+    pos(m);
+  }
+  V vm = vmax(v[0], v[4]);
+  if (!fits(vm)) return false;
+  V nk, qm, qp;
+  stencil(0, nk, qm, qp);
 #pragma unroll
   for (int p = 0; p < K; ++p) {
-    V nm1, rm1, np, rp;
-    if (p + 1 < K) stencil(p + 1, std::true_type{}, std::true_type{}, nm1, rm1, np, rp);
-    else stencil(p + 1, std::false_type{}, std::true_type{}, nm1, rm1, np, rp);
-    w.emit_node(p, c, nm, rm, np, rp, emit);
-    nm = nm1;
-    rm = rm1;
-    if (p + 1 < K) {
-      w.u[p + 6] = u_at(p + 6);
-      pos(p + 6);
-      S[p + 5] = sq(w.D2[p + 5]);
-      al_qX(p + 4);
-      al_qY(p + 4);
-      al_qZ(p + 5);
-    }
+    v[p + 5] = v_at(p + 5);
+    pos(p + 5);
+    V nk1, qm1, qp1;
+    stencil(p + 1, nk1, qm1, qp1);
+    const V mid = vmul(c(0.5f), vadd(v[p + 2], v[p + 3]));
+    const V lm = vfma(c(1.0f / 30.0f), W[p + 1], vfma(c(-0.15f), W[p + 2], vfma(c(-0.05f), W[p + 3], mid)));
+    const V lp = vfma(c(1.0f / 30.0f), W[p + 4], vfma(c(-0.15f), W[p + 3], vfma(c(-0.05f), W[p + 2], mid)));
+    emit(p, vfma(nk, qm, lm), vfma(nk1, qp1, lp));
+    nk = nk1;
+    qm = qm1;
   }
-  return __all_sync(0xffffffffu, ok);
+  return fits(vmax(vm, v[K + 4]));
 }
 
 }  // namespace alw
