@@ -40,12 +40,12 @@ struct Stage2DParams {
   InstDesc inst0;
 };
 
-// TMA box of one tile with its halo (floats): 72 columns x 38 rows for the 64 x 32 tile, 40 x 38
-// for the narrow 32 x 32 tile (batches may choose it).  Padded arrays are laid out for 64-wide
+// TMA box of one tile with its halo (floats): 76 columns x 38 rows for the 64 x 32 tile, 44 x 38
+// for the narrow 32 x 32 tile (batches may choose it); its last columns may lie beyond the array (filled with 0).  Padded arrays are laid out for 64-wide
 // tiles, which also covers the narrow ones.
-constexpr int kBox2DW = 72, kBox2DH = 38;
+constexpr int kBox2DW = 76, kBox2DH = 38;
 constexpr int kTile2DX = 64, kTile2DY = 32;
-constexpr int kTile2DXNarrow = 32, kBox2DWNarrow = 40;
+constexpr int kTile2DXNarrow = 32, kBox2DWNarrow = 44;
 
 // CTAs a launch of `ntiles` work-list entries uses: min(ntiles, grid_ctas or cap, cap).
 inline int stage2d_grid(int ntiles, int grid_ctas, int cap) {

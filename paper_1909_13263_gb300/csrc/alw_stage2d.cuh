@@ -34,141 +34,115 @@
 
 namespace alw {
 
-// Hamiltonians of the 2D examples in float (compile-time kind).  value_sums takes the sums
-// su = u^- + u^+, sv = v^- + v^+ (the Lax-Friedrichs flux evaluates H at (su/2, sv/2)); kSameAlpha
-// marks Hamiltonians whose node alpha is the same in both directions.
+// Hamiltonians of the 2D examples in float (compile-time kind), from the sums and differences of a node's
+// one-sided derivatives, Sx = u^+ + u^-, Dx = u^+ - u^-, Sy = v^+ + v^-, Dy = v^+ - v^-: value is H at the mean
+// derivatives, alpha the maximum of |H_p| and |H_q| over the four corners.  u^-+ = (Sx -+ Dx)/2, so the corner
+// sums u + v are (Sx + Sy)/2 +- (Dx + Dy)/2 and +- (Dx - Dy)/2, and the largest and smallest |u| are
+// (|Sx| +- |Dx|)/2 in magnitude.
 template <int H> struct Ham2;
 template <> struct Ham2<H_BURGERS2D> {
   static constexpr bool kSameAlpha = true;
-  __device__ __forceinline__ static float value(float p, float q, float, float) {
-    const float z = p + q + 1.0f;
-    return 0.5f * z * z;
+  __device__ __forceinline__ static float value(float su, float sv, float, float) {
+    const float z = fmaf(0.353553390593274f, su + sv, 0.707106781186548f);   // ((su + sv)/2 + 1) / sqrt 2
+    return z * z;
   }
-  __device__ __forceinline__ static float value_sums(float su, float sv, float, float) {
-    const float z = fmaf(0.5f, su + sv, 1.0f);
-    return 0.5f * z * z;
-  }
-  __device__ __forceinline__ static void alpha(float um, float up, float vm, float vp, float, float, float &ax,
-                                                    float &ay) {
-    // |H_p| = |H_q| = |u + v + 1| at the four corners: the largest and the smallest corner sums are
-    // max(u) + 1 + max(v) and min(u) + 1 + min(v), and |.| is largest at one of them (the same
-    // values as the four corner sums, with the comparisons on the integer/logic pipe)
-    const float hi = (fmaxf(um, up) + 1.0f) + fmaxf(vm, vp), lo = (fminf(um, up) + 1.0f) + fminf(vm, vp);
-    ax = ay = fmaxf(fabsf(hi), fabsf(lo));
+  // |H_p| = |H_q| = |u + v + 1|: at the largest or the smallest corner sum, (s +- e)/2
+  __device__ __forceinline__ static void alpha(float sx, float dx, float sy, float dy, float, float, float &ax,
+                                               float &ay) {
+    const float s = sx + sy, e = fabsf(dx) + fabsf(dy);
+    ax = ay = fmaxf(fmaf(0.5f, s + e, 1.0f), fmaf(0.5f, e - s, -1.0f));
   }
 };
+// largest |f| over the four corner sums c +- (dx + dy)/2, c +- (dx - dy)/2
+template <class F>
+__device__ __forceinline__ float corner_max(float c, float dx, float dy, F f) {
+  const float p = dx + dy, m = dx - dy;
+  return fmaxf(fmaxf(fabsf(f(fmaf(-0.5f, p, c))), fabsf(f(fmaf(-0.5f, m, c)))),
+               fmaxf(fabsf(f(fmaf(0.5f, m, c))), fabsf(f(fmaf(0.5f, p, c)))));
+}
 template <> struct Ham2<H_NEGCOS2D> {
   static constexpr bool kSameAlpha = true;
-  __device__ __forceinline__ static float value(float p, float q, float, float) { return -sfu_cos(p + q + 1.0f); }
-  __device__ __forceinline__ static float value_sums(float su, float sv, float, float) {
+  __device__ __forceinline__ static float value(float su, float sv, float, float) {
     return -sfu_cos(fmaf(0.5f, su + sv, 1.0f));
   }
-  __device__ __forceinline__ static void alpha(float um, float up, float vm, float vp, float, float, float &ax,
-                                                    float &ay) {
-    const float a = fabsf(sfu_sin(um + vm + 1.0f)), b = fabsf(sfu_sin(um + vp + 1.0f));
-    const float c = fabsf(sfu_sin(up + vm + 1.0f)), d = fabsf(sfu_sin(up + vp + 1.0f));
-    ax = ay = fmaxf(fmaxf(a, b), fmaxf(c, d));
+  __device__ __forceinline__ static void alpha(float sx, float dx, float sy, float dy, float, float, float &ax,
+                                               float &ay) {
+    ax = ay = corner_max(fmaf(0.5f, sx + sy, 1.0f), dx, dy, [](float z) { return sfu_sin(z); });
   }
 };
 template <> struct Ham2<H_SIN2D> {
   static constexpr bool kSameAlpha = true;
-  __device__ __forceinline__ static float value(float p, float q, float, float) { return sfu_sin(p + q); }
-  __device__ __forceinline__ static float value_sums(float su, float sv, float, float) {
-    return sfu_sin(0.5f * (su + sv));
-  }
-  __device__ __forceinline__ static void alpha(float um, float up, float vm, float vp, float, float, float &ax,
-                                                    float &ay) {
-    const float a = fabsf(sfu_cos(um + vm)), b = fabsf(sfu_cos(um + vp));
-    const float c = fabsf(sfu_cos(up + vm)), d = fabsf(sfu_cos(up + vp));
-    ax = ay = fmaxf(fmaxf(a, b), fmaxf(c, d));
+  __device__ __forceinline__ static float value(float su, float sv, float, float) { return sfu_sin(0.5f * (su + sv)); }
+  __device__ __forceinline__ static void alpha(float sx, float dx, float sy, float dy, float, float, float &ax,
+                                               float &ay) {
+    ax = ay = corner_max(0.5f * (sx + sy), dx, dy, [](float z) { return sfu_cos(z); });
   }
 };
 template <> struct Ham2<H_EIKONAL2D> {
   static constexpr bool kSameAlpha = false;
-  __device__ __forceinline__ static float value_sums(float su, float sv, float x, float y) {
-    return value(0.5f * su, 0.5f * sv, x, y);
-  }
-  __device__ __forceinline__ static float value(float p, float q, float, float) {
-    const float t = fmaf(p, p, fmaf(q, q, 1.0f));   // >= 1
+  __device__ __forceinline__ static float value(float su, float sv, float, float) {
+    const float p = 0.5f * su, q = 0.5f * sv, t = fmaf(p, p, fmaf(q, q, 1.0f));   // >= 1
     return t * sfu_rsqrt(t);
   }
-  __device__ __forceinline__ static void alpha(float um, float up, float vm, float vp, float, float, float &ax,
-                                                    float &ay) {
-    const float r00 = sfu_rsqrt(fmaf(um, um, fmaf(vm, vm, 1.0f))), r01 = sfu_rsqrt(fmaf(um, um, fmaf(vp, vp, 1.0f)));
-    const float r10 = sfu_rsqrt(fmaf(up, up, fmaf(vm, vm, 1.0f))), r11 = sfu_rsqrt(fmaf(up, up, fmaf(vp, vp, 1.0f)));
-    ax = fmaxf(fmaxf(fabsf(um) * r00, fabsf(um) * r01), fmaxf(fabsf(up) * r10, fabsf(up) * r11));
-    ay = fmaxf(fmaxf(fabsf(vm) * r00, fabsf(vp) * r01), fmaxf(fabsf(vm) * r10, fabsf(vp) * r11));
+  __device__ __forceinline__ static void alpha(float sx, float dx, float sy, float dy, float, float, float &ax,
+                                               float &ay) {
+    // |H_p| = |u| / sqrt(u^2 + v^2 + 1) grows with |u| and falls with |v|
+    const float uh = 0.5f * (fabsf(sx) + fabsf(dx)), ul = 0.5f * (fabsf(sx) - fabsf(dx));
+    const float vh = 0.5f * (fabsf(sy) + fabsf(dy)), vl = 0.5f * (fabsf(sy) - fabsf(dy));
+    ax = uh * sfu_rsqrt(fmaf(uh, uh, fmaf(vl, vl, 1.0f)));
+    ay = vh * sfu_rsqrt(fmaf(vh, vh, fmaf(ul, ul, 1.0f)));
   }
 };
 
 // Example 11 (optimal control): the only Hamiltonian that depends on the node position (x, y).
 template <> struct Ham2<H_OPTCTRL2D> {
   static constexpr bool kSameAlpha = false;
-  __device__ __forceinline__ static float value_sums(float su, float sv, float x, float y) {
-    return value(0.5f * su, 0.5f * sv, x, y);
-  }
-  __device__ __forceinline__ static float value(float p, float q, float x, float y) {
-    const float sx = sfu_sin(x), cx = sfu_cos(x), sy = sfu_sin(y);
+  __device__ __forceinline__ static float value(float su, float sv, float x, float y) {
+    const float p = 0.5f * su, q = 0.5f * sv, sx = sfu_sin(x), cx = sfu_cos(x), sy = sfu_sin(y);
     // sin(y) p + (sin(x) + sign q) q - sin^2(y)/2 - (1 - cos x), with (sign q) q = |q|
     return fmaf(sy, p, fmaf(sx, q, fabsf(q))) - fmaf(0.5f * sy, sy, 1.0f - cx);
   }
-  __device__ __forceinline__ static void alpha(float, float, float vm, float vp, float x, float y, float &ax,
+  __device__ __forceinline__ static void alpha(float, float, float sv, float dv, float x, float y, float &ax,
                                                float &ay) {
-    // H_p = sin y; H_q = sin x + sign q over [min v, max v], both signs when it contains q = 0
-    const float sx = sfu_sin(x), lo = fminf(vm, vp), hi = fmaxf(vm, vp);
+    // H_p = sin y; H_q = sin x + sign q over [min v, max v] = (Sy -+ |Dy|)/2, both signs when it contains q = 0
+    const float sx = sfu_sin(x), lo = sv - fabsf(dv), hi = sv + fabsf(dv);
     ax = fabsf(sfu_sin(y));
     ay = (lo <= 0.0f && hi >= 0.0f) ? fabsf(sx) + 1.0f : fabsf(sx + (lo > 0.0f ? 1.0f : -1.0f));
   }
 };
 
 // The Hamiltonian of a launch: a compile-time kind, or H_RUNTIME, for batches that run instances
-// of several Hamiltonians in one launch: the kind of the tile's instance, dispatched per node (the
-// branch is uniform across a tile, so warps never diverge on it).
+// of several Hamiltonians in one launch: the kind of the tile's instance, dispatched per tile.
 constexpr int H_RUNTIME = -1;
 // Burgers with a grid-wide or fixed flux alpha: the finish loop does not need each node's alpha, only the
-// grid maximum, so it tracks the largest and the negated smallest corner sum without their + 1 and forms
-// max(hi + 1, -(lo + 1)) = max(|hi + 1|, |lo + 1|) once per fold (hi >= lo)
+// grid maximum, so it tracks twice the largest and twice the negated smallest corner sum without their + 1 and
+// forms max(hi + 1, -(lo + 1)) = max(|hi + 1|, |lo + 1|) once per fold (hi >= lo; the same bits as the largest
+// node alpha, the last rounding being monotone)
 constexpr int H_BURGERS2D_GRID = -2;
 template <int H> struct HamSel {
   static constexpr bool kSameAlpha = Ham2<H>::kSameAlpha;
   static constexpr bool kGridFold = false;
-  __device__ __forceinline__ explicit HamSel(int) {}
-  __device__ __forceinline__ float value_sums(float su, float sv, float x, float y) const {
-    return Ham2<H>::value_sums(su, sv, x, y);
+  __device__ __forceinline__ float value(float su, float sv, float x, float y) const {
+    return Ham2<H>::value(su, sv, x, y);
   }
-  __device__ __forceinline__ void alpha(float um, float up, float vm, float vp, float x, float y, float &ax,
+  __device__ __forceinline__ void alpha(float sx, float dx, float sy, float dy, float x, float y, float &ax,
                                         float &ay) const {
-    Ham2<H>::alpha(um, up, vm, vp, x, y, ax, ay);
+    Ham2<H>::alpha(sx, dx, sy, dy, x, y, ax, ay);
   }
 };
-// runtime kind: the position-free 2D Hamiltonians batches take
 template <> struct HamSel<H_BURGERS2D_GRID> : HamSel<H_BURGERS2D> {
   static constexpr bool kGridFold = true;
-  __device__ __forceinline__ explicit HamSel(int k) : HamSel<H_BURGERS2D>(k) {}
 };
+// runtime kind (batches): the finish loop of a tile is that of its instance's kind, chosen once per tile
 template <> struct HamSel<H_RUNTIME> {
   static constexpr bool kSameAlpha = false;
   static constexpr bool kGridFold = false;
-  int kind;
-  __device__ __forceinline__ explicit HamSel(int k) : kind(k) {}
-  __device__ __forceinline__ float value_sums(float su, float sv, float x, float y) const {
-    switch (kind) {
-      case H_BURGERS2D: return Ham2<H_BURGERS2D>::value_sums(su, sv, x, y);
-      case H_NEGCOS2D: return Ham2<H_NEGCOS2D>::value_sums(su, sv, x, y);
-      case H_SIN2D: return Ham2<H_SIN2D>::value_sums(su, sv, x, y);
-      default: return Ham2<H_EIKONAL2D>::value_sums(su, sv, x, y);
-    }
-  }
-  __device__ __forceinline__ void alpha(float um, float up, float vm, float vp, float x, float y, float &ax,
-                                        float &ay) const {
-    switch (kind) {
-      case H_BURGERS2D: Ham2<H_BURGERS2D>::alpha(um, up, vm, vp, x, y, ax, ay); break;
-      case H_NEGCOS2D: Ham2<H_NEGCOS2D>::alpha(um, up, vm, vp, x, y, ax, ay); break;
-      case H_SIN2D: Ham2<H_SIN2D>::alpha(um, up, vm, vp, x, y, ax, ay); break;
-      default: Ham2<H_EIKONAL2D>::alpha(um, up, vm, vp, x, y, ax, ay); break;
-    }
-  }
 };
+
+// Segments of a warp (of 64) that are not near-linear from which the warp sweeps them in full itself; fewer are
+// shared by the CTA node by node.  Example 10 on 1024^2: 24 segments 63.6 us per step, 40 55.4 us (a kink along a
+// grid line fails the 32 segments of one direction).
+constexpr int kWarpSegs = 40;
 
 // Tile geometry of the stage kernel for tiles TXv nodes wide and 32 high (64 or 32 wide): one thread
 // per 8-node row segment and 8-node column segment, so TXv / 8 warps; the TMA box is the tile plus
@@ -178,12 +152,15 @@ struct Geo2D {
   static constexpr int TX = TXv, TY = kTile2DY, K = 8, NT = TX * TY / K;
   static constexpr int MINB = 512 / NT;                 // resident CTAs per SM the registers are sized for
   static constexpr int CG = TX / 32;                    // column groups of 32 in the y sweep
-  static constexpr int SW = TX + 8, SH = TY + 6;        // TMA box (halo 4 columns / 3 rows each side)
+  // TMA box: halo 4 columns left, 8 right (3 are read: the row sweeps read their cells as 16-byte quads, and
+  // with a pitch of 4 (odd number) floats the quads of a warp's rows fall into distinct banks), 3 rows each side
+  static constexpr int SW = TX + 12, SH = TY + 6;
   static constexpr int ARR = ((SH * SW + 31) / 32) * 32; // floats per array slot (128-byte multiple)
-  static constexpr int DXW = TX + 5, DXP = TX + 9;      // x differences: width, odd pitch
-  static constexpr int SUP = TX + 1;                    // phi_x^-/+ pitch in float2
+  static constexpr int SUP = TX + 1;                    // x hand-off pitch in float2
+  static constexpr int kListCap = 2 * NT;               // segments
   template <int NARR> static constexpr size_t smem_bytes() {
-    return 128 + sizeof(float) * (size_t)(2 * NARR * ARR + TY * DXP) + sizeof(float2) * (size_t)TY * SUP;
+    return 128 + sizeof(float) * (size_t)(2 * NARR * ARR) + sizeof(float2) * (size_t)TY * (SUP + TX) +
+           sizeof(unsigned short) * kListCap;
   }
 };
 static_assert(Geo2D<kTile2DX>::SW == kBox2DW && Geo2D<kTile2DX>::SH == kBox2DH, "TMA box must match the tile halo");
@@ -207,7 +184,7 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
   using G = Geo2D<TXv>;
   constexpr int TX = G::TX, TY = G::TY, K = G::K, NT = G::NT;
   constexpr int SW = G::SW, SH = G::SH, ARR = G::ARR;
-  constexpr int DXW = G::DXW, DXP = G::DXP, SUP = G::SUP, CG = G::CG;
+  constexpr int SUP = G::SUP, CG = G::CG;
   constexpr int NARR = (PREC == P_MIXED) ? 3 : 2;
   const StageParams &p = prm.p;
   const bool batch = prm.insts != nullptr;
@@ -221,8 +198,10 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
   // TMA destinations are kept 128-byte aligned (the launch adds 128 bytes of slack)
   unsigned char *smem = smem_dyn + ((128u - (smem_u32(smem_dyn) & 127u)) & 127u);
   float *raw = reinterpret_cast<float *>(smem);            // [2][NARR][ARR]
-  float *dX = raw + 2 * NARR * ARR;                        // [TY][DXP]
-  float2 *su = reinterpret_cast<float2 *>(dX + TY * DXP);  // [TY][SUP] (offset is an even float count)
+  float2 *su = reinterpret_cast<float2 *>(raw + 2 * NARR * ARR);  // [TY][SUP] sums, differences along x
+  float2 *sv = su + TY * SUP;                                     // [TY][TX] along y
+  unsigned short *s_list = reinterpret_cast<unsigned short *>(sv + TY * TX);  // segments left to the full sweep
+  __shared__ int s_nlist;
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ TileInfo s_info[2];
   __shared__ TileInfo s_pinfo;  // thread 0's last prepared tile (per-instance scalars reused while it repeats)
@@ -352,6 +331,7 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     mbar_init(&bars[0], 1);
     mbar_init(&bars[1], 1);
     fence_mbar_init();
+    s_nlist = 0;
     s_pinfo.inst = -1;
     s_info[0].inst = -1;
     s_info[1].inst = -1;
@@ -389,16 +369,12 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
       __syncthreads();
       continue;
     }
-    // every thread waits for the tile's loads itself; no CTA barrier here: the buffers, the tile
-    // records and the phi_x hand-off of the previous tile are rewritten only after the barrier that
-    // follows the differences pass, which every thread reaches after finishing the previous tile
     const bool ok = mbar_wait_bounded(&bars[buf], (phase >> buf) & 1u);
     phase ^= 1u << buf;
 
     const TileInfo &d = s_info[buf];  // this tile's instance fields (shared memory)
     const int nx = d.nx, ny = d.ny, tx0 = d.tx0, ty0 = d.ty0;
     const size_t rbase = (size_t)d.row_off * p.pitch;   // element offset of the instance's rows
-    const HamSel<H> ham(d.ham);
     const float dtf = s_info[buf].dtf, fax = s_info[buf].fax, fay = s_info[buf].fay;
     const float faxh = 0.5f * fax, fayh = 0.5f * fay;
     const float *A = raw + buf * NARR * ARR;
@@ -409,33 +385,9 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     // finish loop)
     const float *X = (PREC == P_MIXED && prm.map_c >= 0) ? C : B;
 
-    // ---- 1. x differences Delta^+ phi / dx, rows by warp, columns by lane (no division, conflict-free)
-    const float rdx1 = d.rdx;
-    {
-      auto cell_diff = [&](int i0, int i1) -> float {
-        if (PREC == P_MIXED) return (A[i1] - A[i0]) + (X[i1] - X[i0]);
-        return A[i1] - A[i0];
-      };
-      // the first TX cells of every row by whole warps, the last DXW - TX cells of all rows together
-      // (a third pass per row would keep only 5 of 32 lanes busy)
-      static_assert(TX % 32 == 0 && DXW - TX < 32, "x-difference row split");
-      for (int r = warp; r < TY; r += NT / 32) {
-#pragma unroll
-        for (int c = lane; c < TX; c += 32) {
-          const int i0 = (r + 3) * SW + c + 1;
-          dX[r * DXP + c] = cell_diff(i0, i0 + 1) * rdx1;
-        }
-      }
-      for (int j = tid; j < TY * (DXW - TX); j += NT) {
-        const int r = j / (DXW - TX), c = TX + j % (DXW - TX);
-        const int i0 = (r + 3) * SW + c + 1;
-        dX[r * DXP + c] = cell_diff(i0, i0 + 1) * rdx1;
-      }
-    }
     if (__syncthreads_or(!ok)) {
-      // a tile load never completed (the differences pass above ran on whatever the buffer held):
-      // flag the instance and stop; the next tile's load is issued only after this barrier, so no
-      // other load is in flight
+      // a tile load never completed: flag the instance and stop; the next tile's load is issued only
+      // after this barrier, so no other load is in flight
       if (tid == 0) atomicOr(&s_info[buf].st->err, 2);
       __syncthreads();
       return;
@@ -447,75 +399,124 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     const bool edge = (tx0 < 3) || (tx0 + TX > nx - 3) || (ty0 < 3) || (ty0 + TY > ny - 3);
     const int colY = (warp % CG) * 32 + lane, segY = warp / CG;
 
-    // ---- 2. both sweeps in one pass: each thread's row segment (x, lane .x of the packed values)
-    // and column segment (y, lane .y) run the same instruction stream
-    float ym[K], yp[K];
+    // ---- 1. both sweeps in one pass: each thread's row segment (x, lane .x of the packed values)
+    // and column segment (y, lane .y) run the same instruction stream; the sums and differences of the
+    // one-sided derivatives go to shared memory
     {
-      const float *vx = dX + lane * DXP + K * warp;
-      // the y differences of the column segment, formed here from the tile arrays like the x
-      // differences of the differences pass (in the same units); u_at is called for m = 0, 1, 2, ... in
-      // order, so each position loads one new row and reuses the previous one
-      const int iy = (K * segY) * SW + colY + 4;
-      const float rdy1 = d.rdy;
+      // first cell (node - 3) of the column segment, and the quad that ends with that of the row segment
+      const int iy = (K * segY) * SW + colY + 4, ix = (lane + 3) * SW + K * warp;
+      const float2 rd = make_float2(d.rdx, d.rdy);
+      // v_at(m), called for m = 0, 1, 2, ... in order: (v, v) = first differences over dx, dy at position m;
+      // the row's cells come as 16-byte quads (conflict-free, see Geo2D), the column's one by one
+      // (consecutive lanes read consecutive columns)
       auto make_vat = [&]() {
-        float pa = A[iy], px = 0.0f;
-        if (PREC == P_MIXED) px = X[iy];
+        auto quad = [](const float *q, int i) { return *reinterpret_cast<const float4 *>(q + i); };
+        float4 qa = quad(A, ix), qx = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float2 pa = make_float2(qa.y, A[iy]), px = make_float2(0.0f, 0.0f);
+        if (PREC == P_MIXED) {
+          qx = quad(X, ix);
+          px = make_float2(qx.y, X[iy]);
+        }
         return [=](int m) mutable {
-          const int i1 = iy + (m + 1) * SW;
-          float dy;
-          if (PREC == P_MIXED) {
-            const float a1 = A[i1], x1 = X[i1];
-            dy = (a1 - pa) + (x1 - px);
-            pa = a1;
-            px = x1;
-          } else {
-            const float a1 = A[i1];
-            dy = a1 - pa;
-            pa = a1;
+          const int k = (m + 2) & 3, i1 = iy + (m + 1) * SW;   // element of the row's quad
+          if (k == 0) {
+            qa = quad(A, ix + m + 2);
+            if (PREC == P_MIXED) qx = quad(X, ix + m + 2);
           }
-          return make_float2(vx[m], dy * rdy1);
+          auto pick = [&](const float4 &q) { return k == 0 ? q.x : k == 1 ? q.y : k == 2 ? q.z : q.w; };
+          const float2 a1 = make_float2(pick(qa), A[i1]);
+          float2 v = vsub(a1, pa);
+          pa = a1;
+          if (PREC == P_MIXED) {
+            const float2 x1 = make_float2(pick(qx), X[i1]);
+            v = vadd(v, vsub(x1, px));
+            px = x1;
+          }
+          return vmul(v, rd);
         };
       };
-      auto emit = [&](int q, float2 dm, float2 dp) {
-        su[lane * SUP + K * warp + q] = make_float2(dm.x, dp.x);
-        ym[q] = dm.y;
-        yp[q] = dp.y;
+      float2 *ox = su + lane * SUP + K * warp, *oy = sv + (K * segY) * TX + colY;
+      auto emit = [&](int q, float2 S, float2 D) {
+        ox[q] = make_float2(S.x, D.x);
+        oy[q * TX] = make_float2(S.y, D.y);
       };
-      SweepConsts<float2> sc;
-      sc.eps4 = make_float2(4.0f * eps * d.rdx * d.rdx, 4.0f * eps * d.rdy * d.rdy);
-      sc.h2 = make_float2(0.5f * d.dx, 0.5f * d.dy);
-      sc.h3 = make_float2(d.dx * (1.0f / 3.0f), d.dy * (1.0f / 3.0f));
-      sc.mh6 = make_float2(d.dx * (-1.0f / 6.0f), d.dy * (-1.0f / 6.0f));
-      // arc length: every warp sweeps with the near-linear form first and sweeps again in full when some
-      // segment of the warp does not qualify (that form then replaces all its results).  Which form
-      // produced a node's values thus depends only on the data of the warp's segments, whose position on
-      // the grid is fixed by the tile width -- not on the order in which tiles or instances are processed,
-      // nor on history: a single solve, a batch, a server round and a resumed checkpoint (all with
-      // 64-wide tiles) choose alike.
+      // the sweeps that give the one-sided derivatives themselves
+      auto emit_pm = [&](int q, float2 dm, float2 dp) { emit(q, vadd(dp, dm), vsub(dp, dm)); };
+      // arc length: the near-linear form first; segments that do not qualify take the full form, swept again by
+      // the warp where at least kWarpSegs fail (coarse grids, the rounding noise of FP32), else entered in a
+      // list whose nodes all threads of the CTA share (a kink crosses few segments of a tile, and the CTA
+      // would wait for their warps).  Both evaluate the same operations, so a node's derivatives depend only
+      // on the data of its 8-node segment, whose position on the grid is the same for both tile widths --
+      // not on the order in which tiles or instances are processed, nor on history: a single solve, a
+      // batch, a server round and a resumed checkpoint agree.
       if constexpr (W == W_ARCLEN) {
-        const float2 rd = make_float2(d.rdx, d.rdy);
         // FP32 stores phi itself: its rounding over dx is what the derivatives carry anyway
         float2 size = make_float2(0.0f, 0.0f);
         if (PREC == P_F32) {
-          const int ix = (lane + 3) * SW + K * warp + 4;
-          size = make_float2(fmaxf(fabsf(A[ix]), fabsf(A[ix + K - 1])) * d.rdx,
+          size = make_float2(fmaxf(fabsf(A[ix + 4]), fabsf(A[ix + K + 3])) * d.rdx,
                              fmaxf(fabsf(A[iy + 3 * SW]), fabsf(A[iy + (K + 2) * SW])) * d.rdy);
         }
         // segments of rows or columns beyond the grid (ragged tiles) do not count
         if (ty0 + lane >= ny || tx0 + K * warp >= nx) size.x = INFINITY;
         if (tx0 + colY >= nx || ty0 + K * segY >= ny) size.y = INFINITY;
-        if (!sweep_stream_near<K, float2>(make_vat(), rd, make_float2(fmaf(d.dx, d.dx, eps), fmaf(d.dy, d.dy, eps)),
-                                          size, emit)) {
-          auto v_at = make_vat();
-          sweep_stream<K, float2>([&](int m) { return vmul(v_at(m), rd); }, sc, emit);
+        const int near = sweep_stream_near<K, float2>(
+            make_vat(), rd, make_float2(fmaf(d.dx, d.dx, eps), fmaf(d.dy, d.dy, eps)), size, emit);
+        if (__any_sync(0xffffffffu, near != 3)) {
+          const bool fx = !(near & 1), fy = !(near & 2);
+          if (__popc(__ballot_sync(0xffffffffu, fx)) + __popc(__ballot_sync(0xffffffffu, fy)) >= kWarpSegs) {
+            SweepConsts<float2> sc;
+            sc.eps4 = make_float2(4.0f * eps * d.rdx * d.rdx, 4.0f * eps * d.rdy * d.rdy);
+            sc.h2 = make_float2(0.5f * d.dx, 0.5f * d.dy);
+            sc.h3 = make_float2(d.dx * (1.0f / 3.0f), d.dy * (1.0f / 3.0f));
+            sc.mh6 = make_float2(d.dx * (-1.0f / 6.0f), d.dy * (-1.0f / 6.0f));
+            // -0, unknown to the assembler: it fuses a packed multiply (or one with a constant zero added) with
+            // a packed add that is its only reader, as at the first and the last position, and the scalar
+            // sweep of the list, where it does not, would differ in the last bit
+            const float2 nz = vsplat(-(float)(p.stage >> 8), rd);
+            auto v_at = make_vat();
+            sweep_stream<K, float2>([&](int m) { return vfma(v_at(m), rd, nz); }, sc,
+                                    [&](int q, float2 dm, float2 dp) {
+                                      const float2 S = vadd(dp, dm), D = vsub(dp, dm);
+                                      if (fx) ox[q] = make_float2(S.x, D.x);
+                                      if (fy) oy[q * TX] = make_float2(S.y, D.y);
+                                    });
+          } else {
+            // entry: line (row or column), segment along it, direction
+            if (fx) s_list[atomicAdd(&s_nlist, 1)] = (unsigned short)((lane * 8 + warp) * 2);
+            if (fy) s_list[atomicAdd(&s_nlist, 1)] = (unsigned short)((colY * 8 + segY) * 2 + 1);
+          }
         }
       } else {
-        sweep_stream_jp<K, float2>(make_vat(), make_float2(eps, eps), emit);
+        sweep_stream_jp<K, float2>(make_vat(), make_float2(eps, eps), emit_pm);
       }
     }
     __syncthreads();
+    if (W == W_ARCLEN && s_nlist > 0) {
+      for (int i = tid; i < s_nlist * K; i += NT) {
+        const int e = s_list[i / K], q = i % K, along_y = e & 1, line = e >> 4, at = ((e >> 1) & 7) * K + q;
+        const int step = along_y ? SW : 1, i0 = along_y ? at * SW + line + 4 : (line + 3) * SW + at + 1;
+        const float rdl = along_y ? d.rdy : d.rdx, dl = along_y ? d.dy : d.dx;
+        SweepConsts<float> sc;
+        sc.eps4 = 4.0f * eps * rdl * rdl;
+        sc.h2 = 0.5f * dl;
+        sc.h3 = dl * (1.0f / 3.0f);
+        sc.mh6 = dl * (-1.0f / 6.0f);
+        sweep_stream<1, float>(
+            [&](int m) {
+              const int j = i0 + m * step;
+              float v = vsub(A[j + step], A[j]);
+              if (PREC == P_MIXED) v = vadd(v, vsub(X[j + step], X[j]));
+              return vmul(vmul(v, rdl), rdl);
+            },
+            sc, [&](int, float dm, float dp) {
+              (along_y ? sv[at * TX + line] : su[line * SUP + at]) = make_float2(vadd(dp, dm), vsub(dp, dm));
+            });
+      }
+      __syncthreads();
+      if (tid == 0) s_nlist = 0;   // the next entries are made after the next tile's first barrier
+    }
 
-    // ---- 3. nodes (colY, K*segY + q): Lax-Friedrichs Hamiltonian, RK combination, store; one
+    // ---- 2. nodes (colY, K*segY + q): Lax-Friedrichs Hamiltonian, RK combination, store; one
     // unrolled loop per stage and per edge/interior tile, so that no node tests either
     auto finish = [&](auto stage_c, auto edge_c, auto hsel) {
       using HS = decltype(hsel);
@@ -523,26 +524,27 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
       constexpr bool EDGE = decltype(edge_c)::value;
 #pragma unroll
       for (int q = 0; q < K; ++q) {
-        const float dmq = ym[q], dpq = yp[q];
         const int y = K * segY + q;
+        const float2 w = sv[y * TX + colY];    // (Sy, Dy)
+        const float sy = w.x, dy = w.y;
         const int gi = tx0 + colY, gj = ty0 + y;
         const bool inside = !EDGE || (gi < nx && gj < ny);
-        const float2 u = su[y * SUP + colY];
-        const float xn = fmaf((float)gi, d.dx, d.xlo), yn = fmaf((float)gj, d.dy, d.ylo);
-        const float Hv = hsel.value_sums(u.y + u.x, dpq + dmq, xn, yn);
-        float L;
+        const float2 u = su[y * SUP + colY];   // (Sx, Dx)
+        float L;   // -H + alpha_x/2 Dx + alpha_y/2 Dy
         if constexpr (HS::kGridFold) {
-          L = fmaf(faxh, u.y - u.x, fmaf(fayh, dpq - dmq, -Hv));
+          const float s = u.x + sy, e = fabsf(u.y) + fabsf(dy);
+          L = fmaf(faxh, u.y, fmaf(fayh, dy, -hsel.value(u.x, sy, 0.0f, 0.0f)));
           if (inside) {
             nfin = fmaf(L, 0.0f, nfin);
-            amx = fmaxf(amx, fmaxf(u.x, u.y) + fmaxf(dmq, dpq));
-            amy = fmaxf(amy, -(fminf(u.x, u.y) + fminf(dmq, dpq)));
+            amx = fmaxf(amx, s + e);
+            amy = fmaxf(amy, e - s);
           }
         } else {
+          const float xn = fmaf((float)gi, d.dx, d.xlo), yn = fmaf((float)gj, d.dy, d.ylo);
           float ax, ay;
-          hsel.alpha(u.x, u.y, dmq, dpq, xn, yn, ax, ay);
+          hsel.alpha(u.x, u.y, sy, dy, xn, yn, ax, ay);
           const float aX = local_alpha ? ax : fax, aY = local_alpha ? ay : fay;
-          L = fmaf(aX * 0.5f, u.y - u.x, fmaf(aY * 0.5f, dpq - dmq, -Hv));
+          L = fmaf(aX * 0.5f, u.y, fmaf(aY * 0.5f, dy, -hsel.value(u.x, sy, xn, yn)));
           if (inside) {
             // L depends on all four one-sided derivatives: L * 0 is NaN exactly when L is not finite
             nfin = fmaf(L, 0.0f, nfin);
@@ -598,13 +600,13 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     auto finish_h = [&](auto stage_c, auto edge_c) {
       if constexpr (H == H_RUNTIME) {
         switch (d.ham) {
-          case H_BURGERS2D: finish(stage_c, edge_c, HamSel<H_BURGERS2D>(0)); break;
-          case H_NEGCOS2D: finish(stage_c, edge_c, HamSel<H_NEGCOS2D>(0)); break;
-          case H_SIN2D: finish(stage_c, edge_c, HamSel<H_SIN2D>(0)); break;
-          default: finish(stage_c, edge_c, HamSel<H_EIKONAL2D>(0)); break;
+          case H_BURGERS2D: finish(stage_c, edge_c, HamSel<H_BURGERS2D>{}); break;
+          case H_NEGCOS2D: finish(stage_c, edge_c, HamSel<H_NEGCOS2D>{}); break;
+          case H_SIN2D: finish(stage_c, edge_c, HamSel<H_SIN2D>{}); break;
+          default: finish(stage_c, edge_c, HamSel<H_EIKONAL2D>{}); break;
         }
       } else {
-        finish(stage_c, edge_c, ham);
+        finish(stage_c, edge_c, HamSel<H>{});
       }
     };
     auto finish_stage = [&](auto stage_c) {
@@ -623,14 +625,12 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     ++run_tiles;
     const bool more = next < ntiles;
     if (more && !s_info[buf ^ 1].skip && s_info[buf ^ 1].inst == i_inst) {
-      // no barrier: the next tile's differences pass writes only dX, which this tile read
-      // before the barrier after the sweeps; su, raw[buf] and s_info[buf] are rewritten only
-      // after the next tile's barrier that follows its differences pass, which every thread
-      // reaches after finishing this tile
+      // no barrier: su, raw[buf] and s_info[buf] are rewritten only after the next tile's first
+      // barrier, which every thread reaches after finishing this tile
       continue;
     }
     if constexpr (GF) {
-      amx = fmaxf(fmaxf(amx + 1.0f, amy - 1.0f), 0.0f);
+      amx = fmaxf(fmaxf(fmaf(0.5f, amx, 1.0f), fmaf(0.5f, amy, -1.0f)), 0.0f);
       amy = amx;
     } else if (HamSel<H>::kSameAlpha) {
       amy = amx;
@@ -685,7 +685,7 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     amx = amy = A0;
     nfin = 0.0f;
     run_tiles = 0;
-    __syncthreads();  // raw[buf], dX, su, s_info[buf] are free for the next tile
+    __syncthreads();  // raw[buf], su, s_info[buf] are free for the next tile
   }
 }
 

@@ -42,9 +42,8 @@
 // of the weights (0.04 T^3), of the indicators (0.01 T^3) and the interval widths' share of them
 // (0.01 T^2 W + 0.0025 T^2 W^2).  The segment qualifies when that is at most 2^-25 of its largest difference
 // (half a unit of the derivatives' own rounding), or, for a phi stored in float, 2^-25 of |phi| / dx (the
-// rounding of phi itself).  |y|/(y^2 + dx^2) <= 1/(2 dx), whence the bounds hold for any y.  A warp whose
-// segments do not all qualify sweeps them again with sweep_stream; the choice depends on the segments' own
-// data only.
+// rounding of phi itself).  |y|/(y^2 + dx^2) <= 1/(2 dx), whence the bounds hold for any y.  Other
+// segments are swept with sweep_stream; the choice depends on the segment's own data only.
 #pragma once
 #include <type_traits>
 
@@ -402,14 +401,37 @@ __device__ __forceinline__ void sweep_stream_jp(LoadV v_at, V eps, Emit emit) {
   }
 }
 
+// Whether a segment is near-linear: from its largest |T|, |W| and |v| (units of v = Delta^+ phi / dx) and size, what errors
+// are measured against besides |v| (0, or |phi| / dx).  wm: the largest of widths sampled every third position.
+template <class V>
+__device__ __forceinline__ int near_mask(V tm, V wm, V vm, V rdx, V size) {
+  using LN = Lanes<V>;
+  const V t = vmul(tm, rdx), w = vfma(wm, rdx, t);        // |W| <= the nearest sample + |T|
+  const V f = vfma(w, vfma(vsplat(0.0025f, t), w, vsplat(0.01f, t)), vmul(vsplat(0.05f, t), t));
+  const V en = vmul(vmul(tm, t), f);                      // units of v
+  int near = 0;
+#pragma unroll
+  for (int i = 0; i < LN::n; ++i)
+    near |= LN::get(en, i) <= kNearTol * fmaxf(LN::get(vm, i), LN::get(size, i)) ? 1 << i : 0;
+  return near;
+}
+template <class V>
+__device__ __forceinline__ V vmax_abs(V a, V b) {
+  using LN = Lanes<V>;
+  V r;
+#pragma unroll
+  for (int i = 0; i < LN::n; ++i) LN::at(r, i) = fmaxf(fabsf(LN::get(a, i)), fabsf(LN::get(b, i)));
+  return r;
+}
+
 // Near-linear arc-length sweep (see the header comment), in units of the first differences: v_at(m) returns
-// v = Delta^+ phi / dx at position i0 - 3 + m; rdx per lane; e1 = dx^2 + eps; size: what errors are measured
-// against besides the segment's |v| (0, or |phi| / dx).  Called by all 32 threads of a warp; returns, uniformly
-// across the warp, whether every segment of the warp (both lanes of all threads) qualified (checked after
-// the first stencil, where a failing warp stops at once, and after the last).  When it returns false
-// the emitted values, if any, are not to be used and the caller sweeps the warp's segments with sweep_stream.
+// v = Delta^+ phi / dx at position i0 - 3 + m; rdx per lane; e1 = dx^2 + eps; size: see near_mask.  emit(p, S, D)
+// receives the sum and the difference phi^+ +- phi^- of node i0 + p.  Called by all 32 threads of a warp;
+// returns the thread's mask of segments (bit 0: .x, bit 1: .y) that qualified; the emitted values of the
+// others are not to be used.  When no segment of the warp can qualify it stops at once or after the first
+// stencil.
 template <int K, class V, class LoadV, class Emit>
-__device__ __forceinline__ bool sweep_stream_near(LoadV v_at, V rdx, V e1, V size, Emit emit) {
+__device__ __forceinline__ int sweep_stream_near(LoadV v_at, V rdx, V e1, V size, Emit emit) {
   using LN = Lanes<V>;
   V v[K + 5], D[K + 5], W[K + 5], T[K + 5], TT[K + 5];   // TT_m = T_m^2
   V tm = vsplat(0.0f, e1);                               // largest |T|
@@ -424,7 +446,7 @@ __device__ __forceinline__ bool sweep_stream_near(LoadV v_at, V rdx, V e1, V siz
       for (int i = 0; i < LN::n; ++i) LN::at(tm, i) = fmaxf(LN::get(tm, i), fabsf(LN::get(T[m - 1], i)));
     }
   };
-  // stencil j: -k of the "-" side and both quadratic forms
+  // stencil j: -k and both quadratic forms ("+": negated)
   auto stencil = [&](int j, V &nk, V &qm, V &qp) {
     const V y = vfma(c(0.5f), W[j + 2], D[j + 2]);
     const V e = vfma(y, y, e1);
@@ -436,37 +458,24 @@ __device__ __forceinline__ bool sweep_stream_near(LoadV v_at, V rdx, V e1, V siz
     qm = vfma(c(0.06f), TT[j + 2], vfma(c(0.07f), TT[j + 3], vmul(c(-0.03f), ab)));
     qp = vfma(c(-0.07f), TT[j + 2], vfma(c(-0.06f), TT[j + 3], vmul(c(0.03f), ab)));
   };
-  // what the segment's largest T and W leave out, against its size
-  auto fits = [&](V vm) {
-    const V t = vmul(tm, rdx);
-    V w;                                                  // |W| <= |W_1| + 12 |T|
+  // Both early tests count too, so that stopping at them changes no segment's outcome.  A phi stored in float
+  // whose rounding is n = 2^-25 |phi| / dx^2 gives T of 12 to 17 n (measured), which misses the bound where
+  // 0.05 T^3 > n.
+  int begun = 0;
 #pragma unroll
-    for (int i = 0; i < LN::n; ++i) LN::at(w, i) = fabsf(LN::get(W[1], i)) * LN::get(rdx, i);
-    w = vfma(c(12.0f), t, w);
-    const V f = vfma(w, vfma(c(0.0025f), w, c(0.01f)), vmul(c(0.05f), t));
-    const V lhs = vmul(vmul(tm, t), f);                   // T^2 / dx (...) in units of v
-    bool ok = true;
-#pragma unroll
-    for (int i = 0; i < LN::n; ++i) {
-      const float ref = fmaxf(LN::get(vm, i), LN::get(size, i));
-      ok &= LN::get(lhs, i) <= kNearTol * ref;
-    }
-    return __all_sync(0xffffffffu, ok);
-  };
-  auto vmax = [&](V a, V b) {
-    V r;
-#pragma unroll
-    for (int i = 0; i < LN::n; ++i) LN::at(r, i) = fmaxf(fabsf(LN::get(a, i)), fabsf(LN::get(b, i)));
-    return r;
-  };
-
+  for (int i = 0; i < LN::n; ++i) {
+    const float n = kNearTol * LN::get(size, i) * LN::get(rdx, i);
+    begun |= n > 0.04f && n < INFINITY ? 0 : 1 << i;
+  }
+  if (!__any_sync(0xffffffffu, begun != 0)) return 0;
 #pragma unroll
   for (int m = 0; m <= 4; ++m) {
     v[m] = v_at(m);
     pos(m);
   }
-  V vm = vmax(v[0], v[4]);
-  if (!fits(vm)) return false;
+  const V vm = vmax_abs(v[0], v[4]);
+  begun &= near_mask(tm, vmax_abs(W[2], W[2]), vm, rdx, size);
+  if (!__any_sync(0xffffffffu, begun != 0)) return 0;
   V nk, qm, qp;
   stencil(0, nk, qm, qp);
 #pragma unroll
@@ -475,14 +484,15 @@ __device__ __forceinline__ bool sweep_stream_near(LoadV v_at, V rdx, V e1, V siz
     pos(p + 5);
     V nk1, qm1, qp1;
     stencil(p + 1, nk1, qm1, qp1);
-    const V mid = vmul(c(0.5f), vadd(v[p + 2], v[p + 3]));
-    const V lm = vfma(c(1.0f / 30.0f), W[p + 1], vfma(c(-0.15f), W[p + 2], vfma(c(-0.05f), W[p + 3], mid)));
-    const V lp = vfma(c(1.0f / 30.0f), W[p + 4], vfma(c(-0.15f), W[p + 3], vfma(c(-0.05f), W[p + 2], mid)));
-    emit(p, vfma(nk, qm, lm), vfma(nk1, qp1, lp));
+    const V am = vmul(nk, qm), ap = vmul(nk1, qp1);       // what is added to lin^- and lin^+
+    const V s0 = vfma(c(-0.2f), vadd(W[p + 2], W[p + 3]),
+                      vfma(c(1.0f / 30.0f), vadd(W[p + 1], W[p + 4]), vadd(v[p + 2], v[p + 3])));
+    const V d0 = vfma(c(-2.0f), T[p + 3], vadd(T[p + 2], T[p + 4]));   // (lin^+ - lin^-) 30
+    emit(p, vadd(s0, vadd(ap, am)), vfma(c(1.0f / 30.0f), d0, vsub(ap, am)));
     nk = nk1;
     qm = qm1;
   }
-  return fits(vmax(vm, v[K + 4]));
+  return begun & near_mask(tm, vmax_abs(vmax_abs(W[1], W[4]), vmax_abs(W[7], W[10])), vmax_abs(vm, v[K + 4]), rdx, size);
 }
 
 }  // namespace alw
