@@ -33,6 +33,20 @@ static int launch2d_one(const Stage2DParams &prm, cudaStream_t stream) {
   if (cap < 0) return (int)cudaGetLastError();
   const int grid = stage2d_grid(prm.ntiles, prm.grid_ctas, cap);
   if (grid <= 0) return 0;
+  if (prm.nsteps > 0) {
+    // the CTAs wait for one another between stages: a cooperative launch (grid never exceeds what fits)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(G::NT);
+    cfg.dynamicSmemBytes = G::template smem_bytes<NARR>();
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return (int)cudaLaunchKernelEx(&cfg, stage2d_kernel<PREC, W, H, TX>, prm);
+  }
   stage2d_kernel<PREC, W, H, TX><<<grid, G::NT, G::template smem_bytes<NARR>(), stream>>>(prm);
   return (int)cudaGetLastError();
 }

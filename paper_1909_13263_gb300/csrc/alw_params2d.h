@@ -23,6 +23,12 @@ struct InstDesc {
   DevState *st;          // this instance's device-side time and alpha state
 };
 
+// What the CTAs of a launch of several steps share: the barrier's arrivals and the grid maxima per stage.
+struct SoloState {
+  unsigned long long arrived;
+  unsigned long long alpha[3][2];
+};
+
 struct Stage2DParams {
   CUtensorMap maps[6];  // FP32: 0 = phi^n, 1 = stage-1 state, 2 = stage-2 state;
                         // MIXED: 0/1 = hi pairs, 2/3 = lo pairs, 4 = delta_1, 5 = delta_2
@@ -38,6 +44,12 @@ struct Stage2DParams {
   const int *tiles;         // batch: work list, entry = instance * 65536 + tile of that instance
   int *done_count;          // batch: incremented when an instance reaches its t_final (may be null)
   InstDesc inst0;
+  // Whole RK3 steps of the single instance in one cooperative launch (nsteps > 0; lagged or fixed alpha,
+  // periodic): the stage, its maps, output and slots follow from the loop and a grid barrier separates the
+  // stages.  Zero at launch.
+  int nsteps;
+  void *outs[3];
+  SoloState *solo;
 };
 
 // TMA box of one tile with its halo (floats): 76 columns x 38 rows for the 64 x 32 tile, 44 x 38

@@ -144,6 +144,8 @@ struct alw_solver {
   cudaGraphExec_t g_adv = nullptr;
   bool has_phi = false;
   bool line64 = false;      // 1D FP64 grid that fits one cluster: many steps per launch
+  bool multi2d = false;     // periodic 2D float grid: several steps per cooperative launch
+  SoloState *solo = nullptr;  // what their CTAs share
   bool use2d = false;       // persistent TMA kernel (2D float variants)
   int shape64 = 0;          // FP64 2D: tile shape (kShape64)
   CUtensorMap maps[6];      // tensor maps of the padded arrays (see Stage2DParams)
@@ -178,7 +180,18 @@ int kernel_prec(int precision) {
   return precision == ALW_PREC_FP64 ? P_F64 : precision == ALW_PREC_FP32 ? P_F32 : P_MIXED;
 }
 
-int launch_stage(const alw_solver *s, const StageParams &p) {
+// Periodic 2D float grids without a reduction pass before the stage run several steps per cooperative launch, so
+// many that a launch takes a millisecond or two.  The grid barrier between two stages costs less than a kernel's
+// end and the next one's start, at every size; measured (GB300, us per RK3 step of Example 3, a launch per stage
+// -> cooperative): 96^2 35 -> 26, 400^2 28.7 -> 18.5, 1024^2 43.1 -> 33.2, 2048^2 90.4 -> 83.3, 4096^2 279.9 ->
+// 269.8, 8192^2 1004.7 -> 996.1.
+int multi_steps(const alw_solver *s) {
+  const long long n = (1ll << 24) / ((long long)s->nx * s->ny);
+  return n < 4 ? 4 : (n > 64 ? 64 : (int)n);
+}
+
+// nsteps > 0 (2D float): that many whole RK3 steps in one launch instead of the one stage.
+int launch_stage(const alw_solver *s, const StageParams &p, int nsteps = 0) {
   if (s->use2d) {
     Stage2DParams q;
     memset(&q, 0, sizeof q);
@@ -206,6 +219,15 @@ int launch_stage(const alw_solver *s, const StageParams &p) {
     d.lx = s->lx;
     d.ly = s->ly;
     d.st = s->st;
+    if (nsteps > 0) {
+      q.nsteps = nsteps;
+      q.solo = s->solo;
+      q.outs[0] = s->prec == P_MIXED ? s->D1 : s->A;
+      q.outs[1] = s->prec == P_MIXED ? s->D2 : s->B;
+      q.outs[2] = s->prec == P_MIXED ? nullptr : s->P;
+      const cudaError_t e = cudaMemsetAsync(s->solo, 0, sizeof *s->solo, s->stream);
+      if (e != cudaSuccess) return (int)e;
+    }
     const int which = p.stage == 0 ? p.src_of : p.stage;
     if (s->prec == P_MIXED) {
       q.map_a = 0;
@@ -331,6 +353,24 @@ alw_status enqueue_step(alw_solver *s, int loop_mode) {
     ALW_LAUNCH(launch_stage(s, make_params(s, stage, stage, loop_mode)));
     if (linx) ALW_LAUNCH(launch_ghosts(ghost_params(s, stage), s->stream));
   }
+  return ALW_OK;
+}
+
+bool many_steps(const alw_solver *s) { return s->line64 || s->multi2d; }
+int graph_steps(const alw_solver *s) { return s->nx * (long long)s->ny >= (1 << 22) ? 4 : 16; }
+
+// Enqueue n RK3 steps in one launch (the 1D FP64 cluster, or a cooperative launch of the 2D float kernel).  Where
+// the device has no room for the cooperative grid at once (shared or partitioned GPUs), nothing is enqueued and
+// the solver turns to launches per stage.
+alw_status enqueue_many(alw_solver *s, int loop_mode, int n) {
+  const StageParams p = make_params(s, 3, 3, loop_mode);
+  const int e = s->line64 ? launch_line64(p, n, s->stream) : launch_stage(s, p, n);
+  if (s->multi2d && e == (int)cudaErrorCooperativeLaunchTooLarge) {
+    cudaGetLastError();
+    s->multi2d = false;
+    return ALW_OK;
+  }
+  ALW_LAUNCH(e);
   return ALW_OK;
 }
 
@@ -505,6 +545,7 @@ alw_status alw_create(const alw_grid *grid, const alw_hamiltonian *ham, const al
   s->elem = s->prec == P_F64 ? 8 : 4;
   s->use2d = s->dim == 2 && s->prec != P_F64;
   s->line64 = s->dim == 1 && s->prec == P_F64 && s->nx <= kLine64Max && !exact_mode(s->alpha_mode);
+  s->multi2d = s->use2d && !exact_mode(s->alpha_mode) && per;
   s->arr_bytes = (size_t)s->pitch * s->rows * s->elem;
 
   auto cleanup = [&](alw_status st) {
@@ -518,6 +559,8 @@ alw_status alw_create(const alw_grid *grid, const alw_hamiltonian *ham, const al
   }
   s->st = (DevState *)s->alloc(sizeof(DevState));
   if (!s->st) return cleanup(fail(ALW_ENOMEM, "device allocation failed"));
+  if (s->multi2d && !(s->solo = (SoloState *)s->alloc(sizeof *s->solo)))
+    return cleanup(fail(ALW_ENOMEM, "device allocation failed"));
   std::vector<void **> bufs;
   if (s->prec == P_MIXED) bufs = {&s->H[0], &s->H[1], &s->Lo[0], &s->Lo[1], &s->D1, &s->D2};
   else bufs = {&s->P, &s->A, &s->B};
@@ -612,10 +655,10 @@ alw_status alw_step_to(alw_solver *s, double t_final, int64_t *steps_out) {
   alw_status st = check_solver(s);
   if (st) return st;
   if (!std::isfinite(t_final)) return fail(ALW_EINVAL, "t_final must be finite");
-  if (s->line64) {
-    s->g_step_n = kLineSteps;
+  if (many_steps(s)) {
+    s->g_step_n = s->line64 ? kLineSteps : multi_steps(s);
   } else if (!s->g_step) {
-    s->g_step_n = (s->nx * (long long)s->ny >= (1 << 22)) ? 4 : 16;
+    s->g_step_n = graph_steps(s);
     st = build_graph(s, LOOP_STEP_TO, s->g_step_n, &s->g_step);
     if (st) return st;
   }
@@ -634,8 +677,18 @@ alw_status alw_step_to(alw_solver *s, double t_final, int64_t *steps_out) {
     const double t_prev = s->h_st->t;
     const int64_t steps_prev = s->h_st->steps;
     for (int r = 0; r < replays; ++r) {
-      if (s->line64) ALW_LAUNCH(launch_line64(make_params(s, 3, 3, LOOP_STEP_TO), kLineSteps, s->stream));
-      else ALW_CUDA(cudaGraphLaunch(s->g_step, s->stream));
+      if (many_steps(s)) {
+        st = enqueue_many(s, LOOP_STEP_TO, s->g_step_n);
+        if (st) return st;
+        if (!many_steps(s)) {
+          s->g_step_n = graph_steps(s);
+          st = build_graph(s, LOOP_STEP_TO, s->g_step_n, &s->g_step);
+          if (st) return st;
+          break;
+        }
+      } else {
+        ALW_CUDA(cudaGraphLaunch(s->g_step, s->stream));
+      }
     }
     st = read_state(s);
     if (st) return st;
@@ -668,13 +721,13 @@ alw_status alw_advance(alw_solver *s, int64_t nsteps) {
   alw_status st = check_solver(s);
   if (st) return st;
   if (nsteps < 0) return fail(ALW_EINVAL, "nsteps < 0");
-  if (s->line64) {
-    for (int64_t i = 0; i < nsteps; i += kLineSteps) {
-      const int k = (int)(nsteps - i < kLineSteps ? nsteps - i : kLineSteps);
-      ALW_LAUNCH(launch_line64(make_params(s, 3, 3, LOOP_ADVANCE), k, s->stream));
-    }
-    return ALW_OK;
+  while (nsteps > 0 && many_steps(s)) {
+    const int most = s->line64 ? kLineSteps : multi_steps(s), k = (int)(nsteps < most ? nsteps : most);
+    st = enqueue_many(s, LOOP_ADVANCE, k);
+    if (st) return st;
+    if (many_steps(s)) nsteps -= k;
   }
+  if (nsteps == 0) return ALW_OK;
   if (!s->g_adv) {
     st = build_graph(s, LOOP_ADVANCE, 1, &s->g_adv);
     if (st) return st;

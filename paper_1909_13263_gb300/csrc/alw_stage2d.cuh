@@ -1,23 +1,22 @@
 // Persistent 2D stage kernel for float arithmetic (FP32 and MIXED) on sm_103a,
 // for one instance or a batch of instances stacked in shared padded arrays.
 //
-// Each CTA walks the work list (tile = blockIdx.x + k * gridDim.x).  Thread 0
-// prepares the next tile -- decodes its instance, decides whether the instance
+// A launch is one stage, or several whole RK3 steps of one grid with a barrier
+// of the CTAs between stages.  Each CTA walks the work list (tile = blockIdx.x
+// + k * gridDim.x).  Thread 0 prepares the next tile -- decodes its instance, decides whether the instance
 // still needs work, computes the instance's dt and flux alpha for this stage,
 // and issues one TMA box per array (tile plus 3-node halo) into the other half
 // of a double buffer on an mbarrier -- while all threads compute the current
 // tile:
-//   1. differences pass: Delta^+ phi along x (dX) for every cell, combining
-//      the two MIXED parts (hi + lo, or hi + the previous stage's increment
-//      array, which carries lo) once per cell;
-//   2. both sweeps in one pass, packed two lanes per value (f32x2): each
-//      thread sweeps nodes 8w..8w+7 of row `lane` along x (warp w; the odd dX
-//      pitch makes these column-wise reads conflict-free) in lane .x and 8
-//      consecutive nodes of one column along y in lane .y, whose differences
-//      it forms itself from the tile arrays (consecutive lanes read
-//      consecutive columns); phi_x^-/+ go to shared memory, phi_y^-/+ stay in
-//      registers;
-//   3. each thread forms, for its 8 column nodes, the Lax-Friedrichs
+//   1. both sweeps in one pass, packed two lanes per value (f32x2): each
+//      thread sweeps nodes 8w..8w+7 of row `lane` along x (warp w; it reads
+//      its cells as 16-byte quads, which the box pitch keeps conflict-free) in
+//      lane .x and 8 consecutive nodes of one column along y in lane .y
+//      (consecutive lanes read consecutive columns), combining the two MIXED
+//      parts (hi + lo, or hi + the previous stage's increment array, which
+//      carries lo) as it goes; the sums and differences of the one-sided
+//      derivatives go to shared memory;
+//   2. each thread forms, for its 8 column nodes, the Lax-Friedrichs
 //      Hamiltonian and the RK combination, and stores.
 // A CTA keeps running maxima of |dH/dp|, |dH/dq| over consecutive tiles of
 // one instance and folds them into the instance's slot (with the number of
@@ -143,6 +142,8 @@ template <> struct HamSel<H_RUNTIME> {
 // shared by the CTA node by node.  Example 10 on 1024^2: 24 segments 63.6 us per step, 40 55.4 us (a kink along a
 // grid line fails the 32 segments of one direction).
 constexpr int kWarpSegs = 40;
+// Reads of the grid barrier's counter before a CTA gives up (about 0.5 us each).
+constexpr int kBarrierSpins = 1 << 22;
 
 // Tile geometry of the stage kernel for tiles TXv nodes wide and 32 high (64 or 32 wide): one thread
 // per 8-node row segment and 8-node column segment, so TXv / 8 warps; the TMA box is the tile plus
@@ -178,6 +179,11 @@ struct TileInfo {
   DevState *st;
 };
 
+struct SoloLocal {
+  double t, tf, dt, a[2], ends[2][2];   // a: grid maxima of the last stage; ends: of stages 2, 3 of the last whole step
+  int cur, last, err, steps;
+};
+
 template <int PREC, int W, int H, int TXv>
 __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     stage2d_kernel(const __grid_constant__ Stage2DParams prm) {
@@ -188,7 +194,13 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
   constexpr int NARR = (PREC == P_MIXED) ? 3 : 2;
   const StageParams &p = prm.p;
   const bool batch = prm.insts != nullptr;
-  if (!batch) {
+  // one stage, or (solo: a single grid, cooperative launch) prm.nsteps RK3 steps, stage run % 3 + 1 in run `run`.
+  // The CTAs keep a copy of the grid's state each, advanced by the same arithmetic, and meet once per stage: the
+  // maxima and the arrival count are the only global atomics between two stages.
+  const bool solo = prm.nsteps > 0;
+  const int runs = solo ? 3 * prm.nsteps : 1;
+  int stage = p.stage, map_c = prm.map_c;
+  if (!batch && !solo) {
     const DevState *st = prm.inst0.st;
     if (p.loop_mode == LOOP_STEP_TO && !(st->t < st->t_final)) return;
     if (st->err) return;
@@ -201,7 +213,8 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
   float2 *su = reinterpret_cast<float2 *>(raw + 2 * NARR * ARR);  // [TY][SUP] sums, differences along x
   float2 *sv = su + TY * SUP;                                     // [TY][TX] along y
   unsigned short *s_list = reinterpret_cast<unsigned short *>(sv + TY * TX);  // segments left to the full sweep
-  __shared__ int s_nlist;
+  __shared__ int s_nlist, s_stop, s_lost;
+  __shared__ SoloLocal so;   // solo: the instance's state, advanced alike by thread 0 of every CTA
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ TileInfo s_info[2];
   __shared__ TileInfo s_pinfo;  // thread 0's last prepared tile (per-instance scalars reused while it repeats)
@@ -221,10 +234,11 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     if (PREC == P_MIXED) {
       mA = &prm.maps[prm.map_a + info.cur];
       mB = &prm.maps[prm.map_b + info.cur];
-      if (prm.map_c >= 0) mC = &prm.maps[prm.map_c];
+      if (map_c >= 0) mC = &prm.maps[map_c];
     } else {
-      mA = &prm.maps[prm.map_a];
-      if (prm.map_b >= 0) mB = &prm.maps[prm.map_b];
+      // the stage's input (of stage 0: that of the stage p.src_of) and phi^n
+      mA = &prm.maps[stage == 0 ? prm.map_a : stage - 1];
+      if (stage >= 2) mB = &prm.maps[0];
     }
     const int nm = 1 + (mB != nullptr) + (mC != nullptr);
     float *dst = raw + b * NARR * ARR;
@@ -289,7 +303,7 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     info.skip = (s_err != 0) || (p.loop_mode == LOOP_STEP_TO && !(s_t < s_tf));
     double dt;
     int last = 0;
-    if (p.stage == 1 && p.loop_mode != LOOP_STAGE) {
+    if (stage == 1 && p.loop_mode != LOOP_STAGE) {
       double ax, ay;
       if (p.alpha_mode == A_FIXED) {
         ax = p.alpha_fixed[0];
@@ -332,10 +346,6 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
     mbar_init(&bars[1], 1);
     fence_mbar_init();
     s_nlist = 0;
-    s_pinfo.inst = -1;
-    s_info[0].inst = -1;
-    s_info[1].inst = -1;
-    if ((int)blockIdx.x < ntiles) prepare(blockIdx.x, batch ? prm.tiles[blockIdx.x] : 0, 0);
   }
   __syncthreads();
 
@@ -347,8 +357,7 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
   float amx = A0, amy = A0;
   float nfin = 0.0f;  // NaN once a non-finite L was met (see the finish loop)
   int run_tiles = 0;
-  // thread 0: work-list entry of the tile after next, loaded one tile ahead of its use
-  int e_ahead = (batch && tid == 0 && (int)(blockIdx.x + gridDim.x) < ntiles) ? prm.tiles[blockIdx.x + gridDim.x] : 0;
+  int e_ahead = 0;  // thread 0: work-list entry of the tile after next, loaded one tile ahead of its use
   // thread 0, once every thread is past the previous tile's reads of buffer buf ^ 1 and of
   // s_info[buf ^ 1]: prepare the next tile into that buffer
   auto prepare_next = [&](int next, int buf) {
@@ -359,333 +368,460 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
       e_ahead = (batch && after < ntiles) ? prm.tiles[after] : 0;
     }
   };
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++k) {
-    const int buf = k & 1;
-    const int next = t + gridDim.x;
-    const int i_inst = s_info[buf].inst, i_skip = s_info[buf].skip, i_cur = s_info[buf].cur;
-    if (i_skip) {
-      __syncthreads();
-      prepare_next(next, buf);
-      __syncthreads();
-      continue;
+  if (solo && tid == 0) {
+    const DevState *st = prm.inst0.st;
+    so.t = st->t;
+    so.tf = st->t_final;
+    so.dt = st->dt;
+    so.last = st->last;
+    so.cur = st->cur;
+    so.err = st->err;
+    so.steps = 0;
+    for (int i = 0; i < 2; ++i) so.a[i] = bits_to_double(st->alpha_bits[2][i]);
+  }
+  // the stage's first tile: its loads are issued before the scalars are worked out
+  auto prepare_solo = [&](int t, int b) {
+    const InstDesc &d = prm.inst0;
+    TileInfo info;
+    info.inst = 0;
+    info.tiles_x = d.tiles_x;
+    info.tx0 = (t % d.tiles_x) * TX;
+    info.ty0 = (t / d.tiles_x) * TY;
+    info.row_off = d.row_off;
+    info.cur = (PREC == P_MIXED) ? so.cur : 0;
+    info.skip = 0;
+    issue_loads(info, b);
+    info.nx = d.nx;
+    info.ny = d.ny;
+    info.bc = d.bc;
+    info.ham = d.ham;
+    info.ntiles = d.ntiles;
+    info.dx = d.dx;
+    info.dy = d.dy;
+    info.rdx = d.rdx;
+    info.rdy = d.rdy;
+    info.xlo = d.xlo;
+    info.ylo = d.ylo;
+    info.st = d.st;
+    const bool fixed = p.alpha_mode == A_FIXED;
+    if (stage == 1) {
+      const double den = (fixed ? p.alpha_fixed[0] : so.a[0]) / d.lx + (fixed ? p.alpha_fixed[1] : so.a[1]) / d.ly;
+      so.dt = den > 0.0 ? p.cfl / den : (p.loop_mode == LOOP_ADVANCE ? 0.0 : INFINITY);
+      so.last = p.loop_mode == LOOP_STEP_TO && so.t + so.dt >= so.tf;
+      if (so.last) so.dt = so.tf - so.t;
     }
-    const bool ok = mbar_wait_bounded(&bars[buf], (phase >> buf) & 1u);
-    phase ^= 1u << buf;
-
-    const TileInfo &d = s_info[buf];  // this tile's instance fields (shared memory)
-    const int nx = d.nx, ny = d.ny, tx0 = d.tx0, ty0 = d.ty0;
-    const size_t rbase = (size_t)d.row_off * p.pitch;   // element offset of the instance's rows
-    const float dtf = s_info[buf].dtf, fax = s_info[buf].fax, fay = s_info[buf].fay;
-    const float faxh = 0.5f * fax, fayh = 0.5f * fay;
-    const float *A = raw + buf * NARR * ARR;
-    const float *B = A + ARR;
-    const float *C = A + 2 * ARR;
-    // MIXED: the stage's input is A + X, the high part of phi^n plus X = its low part (stage 1) or the
-    // increment array of the previous stage, which holds the low part as well (stages 2 and 3; see the
-    // finish loop)
-    const float *X = (PREC == P_MIXED && prm.map_c >= 0) ? C : B;
-
-    if (__syncthreads_or(!ok)) {
-      // a tile load never completed: flag the instance and stop; the next tile's load is issued only
-      // after this barrier, so no other load is in flight
-      if (tid == 0) atomicOr(&s_info[buf].st->err, 2);
-      __syncthreads();
-      return;
+    info.dt = so.dt;
+    info.dtf = (float)so.dt;
+    info.last = so.last;
+    info.fax = fixed ? (float)p.alpha_fixed[0] : (local_alpha ? 0.0f : (float)so.a[0]);
+    info.fay = fixed ? (float)p.alpha_fixed[1] : (local_alpha ? 0.0f : (float)so.a[1]);
+    s_info[b] = info;
+    s_pinfo = info;
+  };
+  for (int run = 0; run < runs; ++run) {
+    if (solo) {
+      stage = run % 3 + 1;
+      map_c = stage == 1 ? -1 : stage + 2;
     }
-    // every thread has finished the previous tile (its finish loop read buffer buf ^ 1), so the next
-    // tile's load can go there; the barrier after the sweeps publishes s_info[buf ^ 1]
-    prepare_next(next, buf);
-
-    const bool edge = (tx0 < 3) || (tx0 + TX > nx - 3) || (ty0 < 3) || (ty0 + TY > ny - 3);
-    const int colY = (warp % CG) * 32 + lane, segY = warp / CG;
-
-    // ---- 1. both sweeps in one pass: each thread's row segment (x, lane .x of the packed values)
-    // and column segment (y, lane .y) run the same instruction stream; the sums and differences of the
-    // one-sided derivatives go to shared memory
-    {
-      // first cell (node - 3) of the column segment, and the quad that ends with that of the row segment
-      const int iy = (K * segY) * SW + colY + 4, ix = (lane + 3) * SW + K * warp;
-      const float2 rd = make_float2(d.rdx, d.rdy);
-      // v_at(m), called for m = 0, 1, 2, ... in order: (v, v) = first differences over dx, dy at position m;
-      // the row's cells come as 16-byte quads (conflict-free, see Geo2D), the column's one by one
-      // (consecutive lanes read consecutive columns)
-      auto make_vat = [&]() {
-        auto quad = [](const float *q, int i) { return *reinterpret_cast<const float4 *>(q + i); };
-        float4 qa = quad(A, ix), qx = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        float2 pa = make_float2(qa.y, A[iy]), px = make_float2(0.0f, 0.0f);
-        if (PREC == P_MIXED) {
-          qx = quad(X, ix);
-          px = make_float2(qx.y, X[iy]);
-        }
-        return [=](int m) mutable {
-          const int k = (m + 2) & 3, i1 = iy + (m + 1) * SW;   // element of the row's quad
-          if (k == 0) {
-            qa = quad(A, ix + m + 2);
-            if (PREC == P_MIXED) qx = quad(X, ix + m + 2);
-          }
-          auto pick = [&](const float4 &q) { return k == 0 ? q.x : k == 1 ? q.y : k == 2 ? q.z : q.w; };
-          const float2 a1 = make_float2(pick(qa), A[i1]);
-          float2 v = vsub(a1, pa);
-          pa = a1;
-          if (PREC == P_MIXED) {
-            const float2 x1 = make_float2(pick(qx), X[i1]);
-            v = vadd(v, vsub(x1, px));
-            px = x1;
-          }
-          return vmul(v, rd);
-        };
-      };
-      float2 *ox = su + lane * SUP + K * warp, *oy = sv + (K * segY) * TX + colY;
-      auto emit = [&](int q, float2 S, float2 D) {
-        ox[q] = make_float2(S.x, D.x);
-        oy[q * TX] = make_float2(S.y, D.y);
-      };
-      // the sweeps that give the one-sided derivatives themselves
-      auto emit_pm = [&](int q, float2 dm, float2 dp) { emit(q, vadd(dp, dm), vsub(dp, dm)); };
-      // arc length: the near-linear form first; segments that do not qualify take the full form, swept again by
-      // the warp where at least kWarpSegs fail (coarse grids, the rounding noise of FP32), else entered in a
-      // list whose nodes all threads of the CTA share (a kink crosses few segments of a tile, and the CTA
-      // would wait for their warps).  Both evaluate the same operations, so a node's derivatives depend only
-      // on the data of its 8-node segment, whose position on the grid is the same for both tile widths --
-      // not on the order in which tiles or instances are processed, nor on history: a single solve, a
-      // batch, a server round and a resumed checkpoint agree.
-      if constexpr (W == W_ARCLEN) {
-        // FP32 stores phi itself: its rounding over dx is what the derivatives carry anyway
-        float2 size = make_float2(0.0f, 0.0f);
-        if (PREC == P_F32) {
-          size = make_float2(fmaxf(fabsf(A[ix + 4]), fabsf(A[ix + K + 3])) * d.rdx,
-                             fmaxf(fabsf(A[iy + 3 * SW]), fabsf(A[iy + (K + 2) * SW])) * d.rdy);
-        }
-        // segments of rows or columns beyond the grid (ragged tiles) do not count
-        if (ty0 + lane >= ny || tx0 + K * warp >= nx) size.x = INFINITY;
-        if (tx0 + colY >= nx || ty0 + K * segY >= ny) size.y = INFINITY;
-        const int near = sweep_stream_near<K, float2>(
-            make_vat(), rd, make_float2(fmaf(d.dx, d.dx, eps), fmaf(d.dy, d.dy, eps)), size, emit);
-        if (__any_sync(0xffffffffu, near != 3)) {
-          const bool fx = !(near & 1), fy = !(near & 2);
-          if (__popc(__ballot_sync(0xffffffffu, fx)) + __popc(__ballot_sync(0xffffffffu, fy)) >= kWarpSegs) {
-            SweepConsts<float2> sc;
-            sc.eps4 = make_float2(4.0f * eps * d.rdx * d.rdx, 4.0f * eps * d.rdy * d.rdy);
-            sc.h2 = make_float2(0.5f * d.dx, 0.5f * d.dy);
-            sc.h3 = make_float2(d.dx * (1.0f / 3.0f), d.dy * (1.0f / 3.0f));
-            sc.mh6 = make_float2(d.dx * (-1.0f / 6.0f), d.dy * (-1.0f / 6.0f));
-            // -0, unknown to the assembler: it fuses a packed multiply (or one with a constant zero added) with
-            // a packed add that is its only reader, as at the first and the last position, and the scalar
-            // sweep of the list, where it does not, would differ in the last bit
-            const float2 nz = vsplat(-(float)(p.stage >> 8), rd);
-            auto v_at = make_vat();
-            sweep_stream<K, float2>([&](int m) { return vfma(v_at(m), rd, nz); }, sc,
-                                    [&](int q, float2 dm, float2 dp) {
-                                      const float2 S = vadd(dp, dm), D = vsub(dp, dm);
-                                      if (fx) ox[q] = make_float2(S.x, D.x);
-                                      if (fy) oy[q * TX] = make_float2(S.y, D.y);
-                                    });
-          } else {
-            // entry: line (row or column), segment along it, direction
-            if (fx) s_list[atomicAdd(&s_nlist, 1)] = (unsigned short)((lane * 8 + warp) * 2);
-            if (fy) s_list[atomicAdd(&s_nlist, 1)] = (unsigned short)((colY * 8 + segY) * 2 + 1);
-          }
-        }
-      } else {
-        sweep_stream_jp<K, float2>(make_vat(), make_float2(eps, eps), emit_pm);
+    if (tid == 0) {
+      s_pinfo.inst = s_info[0].inst = s_info[1].inst = -1;
+      s_stop = solo && (so.err || (stage == 1 && p.loop_mode == LOOP_STEP_TO && !(so.t < so.tf)));
+      if (!s_stop && (int)blockIdx.x < ntiles) {
+        fence_proxy_async_smem();
+        if (solo) prepare_solo(blockIdx.x, k & 1);
+        else prepare(blockIdx.x, batch ? prm.tiles[blockIdx.x] : 0, k & 1);
+        e_ahead = (batch && (int)(blockIdx.x + gridDim.x) < ntiles) ? prm.tiles[blockIdx.x + gridDim.x] : 0;
+        // the next stage's maxima: last read in the stage before this one
+        if (solo && blockIdx.x == 0) prm.solo->alpha[stage % 3][0] = prm.solo->alpha[stage % 3][1] = 0ull;
       }
     }
     __syncthreads();
-    if (W == W_ARCLEN && s_nlist > 0) {
-      for (int i = tid; i < s_nlist * K; i += NT) {
-        const int e = s_list[i / K], q = i % K, along_y = e & 1, line = e >> 4, at = ((e >> 1) & 7) * K + q;
-        const int step = along_y ? SW : 1, i0 = along_y ? at * SW + line + 4 : (line + 3) * SW + at + 1;
-        const float rdl = along_y ? d.rdy : d.rdx, dl = along_y ? d.dy : d.dx;
-        SweepConsts<float> sc;
-        sc.eps4 = 4.0f * eps * rdl * rdl;
-        sc.h2 = 0.5f * dl;
-        sc.h3 = dl * (1.0f / 3.0f);
-        sc.mh6 = dl * (-1.0f / 6.0f);
-        sweep_stream<1, float>(
-            [&](int m) {
-              const int j = i0 + m * step;
-              float v = vsub(A[j + step], A[j]);
-              if (PREC == P_MIXED) v = vadd(v, vsub(X[j + step], X[j]));
-              return vmul(vmul(v, rdl), rdl);
-            },
-            sc, [&](int, float dm, float dp) {
-              (along_y ? sv[at * TX + line] : su[line * SUP + at]) = make_float2(vadd(dp, dm), vsub(dp, dm));
-            });
+    if (s_stop) break;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++k) {
+      const int buf = k & 1;
+      const int next = t + gridDim.x;
+      const int i_inst = s_info[buf].inst, i_skip = s_info[buf].skip, i_cur = s_info[buf].cur;
+      if (i_skip) {
+        __syncthreads();
+        prepare_next(next, buf);
+        __syncthreads();
+        continue;
       }
-      __syncthreads();
-      if (tid == 0) s_nlist = 0;   // the next entries are made after the next tile's first barrier
-    }
+      const bool ok = mbar_wait_bounded(&bars[buf], (phase >> buf) & 1u);
+      phase ^= 1u << buf;
 
-    // ---- 2. nodes (colY, K*segY + q): Lax-Friedrichs Hamiltonian, RK combination, store; one
-    // unrolled loop per stage and per edge/interior tile, so that no node tests either
-    auto finish = [&](auto stage_c, auto edge_c, auto hsel) {
-      using HS = decltype(hsel);
-      constexpr int ST = decltype(stage_c)::value;
-      constexpr bool EDGE = decltype(edge_c)::value;
-#pragma unroll
-      for (int q = 0; q < K; ++q) {
-        const int y = K * segY + q;
-        const float2 w = sv[y * TX + colY];    // (Sy, Dy)
-        const float sy = w.x, dy = w.y;
-        const int gi = tx0 + colY, gj = ty0 + y;
-        const bool inside = !EDGE || (gi < nx && gj < ny);
-        const float2 u = su[y * SUP + colY];   // (Sx, Dx)
-        float L;   // -H + alpha_x/2 Dx + alpha_y/2 Dy
-        if constexpr (HS::kGridFold) {
-          const float s = u.x + sy, e = fabsf(u.y) + fabsf(dy);
-          L = fmaf(faxh, u.y, fmaf(fayh, dy, -hsel.value(u.x, sy, 0.0f, 0.0f)));
-          if (inside) {
-            nfin = fmaf(L, 0.0f, nfin);
-            amx = fmaxf(amx, s + e);
-            amy = fmaxf(amy, e - s);
+      const TileInfo &d = s_info[buf];  // this tile's instance fields (shared memory)
+      const int nx = d.nx, ny = d.ny, tx0 = d.tx0, ty0 = d.ty0;
+      const size_t rbase = (size_t)d.row_off * p.pitch;   // element offset of the instance's rows
+      const float dtf = s_info[buf].dtf, fax = s_info[buf].fax, fay = s_info[buf].fay;
+      const float faxh = 0.5f * fax, fayh = 0.5f * fay;
+      const float *A = raw + buf * NARR * ARR;
+      const float *B = A + ARR;
+      const float *C = A + 2 * ARR;
+      // MIXED: the stage's input is A + X, the high part of phi^n plus X = its low part (stage 1) or the
+      // increment array of the previous stage, which holds the low part as well (stages 2 and 3; see the
+      // finish loop)
+      const float *X = (PREC == P_MIXED && map_c >= 0) ? C : B;
+
+      if (__syncthreads_or(!ok)) {
+        // a tile load never completed: flag the instance and stop; the next tile's load is issued only
+        // after this barrier, so no other load is in flight
+        if (tid == 0) atomicOr(&s_info[buf].st->err, 2);
+        __syncthreads();
+        return;
+      }
+      // every thread has finished the previous tile (its finish loop read buffer buf ^ 1), so the next
+      // tile's load can go there; the barrier after the sweeps publishes s_info[buf ^ 1]
+      prepare_next(next, buf);
+
+      const bool edge = (tx0 < 3) || (tx0 + TX > nx - 3) || (ty0 < 3) || (ty0 + TY > ny - 3);
+      const int colY = (warp % CG) * 32 + lane, segY = warp / CG;
+
+      // ---- 1. both sweeps in one pass: each thread's row segment (x, lane .x of the packed values)
+      // and column segment (y, lane .y) run the same instruction stream; the sums and differences of the
+      // one-sided derivatives go to shared memory
+      {
+        // first cell (node - 3) of the column segment, and the quad that ends with that of the row segment
+        const int iy = (K * segY) * SW + colY + 4, ix = (lane + 3) * SW + K * warp;
+        const float2 rd = make_float2(d.rdx, d.rdy);
+        // v_at(m), called for m = 0, 1, 2, ... in order: (v, v) = first differences over dx, dy at position m;
+        // the row's cells come as 16-byte quads (conflict-free, see Geo2D), the column's one by one
+        // (consecutive lanes read consecutive columns)
+        auto make_vat = [&]() {
+          auto quad = [](const float *q, int i) { return *reinterpret_cast<const float4 *>(q + i); };
+          float4 qa = quad(A, ix), qx = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          float2 pa = make_float2(qa.y, A[iy]), px = make_float2(0.0f, 0.0f);
+          if (PREC == P_MIXED) {
+            qx = quad(X, ix);
+            px = make_float2(qx.y, X[iy]);
+          }
+          return [=](int m) mutable {
+            const int k = (m + 2) & 3, i1 = iy + (m + 1) * SW;   // element of the row's quad
+            if (k == 0) {
+              qa = quad(A, ix + m + 2);
+              if (PREC == P_MIXED) qx = quad(X, ix + m + 2);
+            }
+            auto pick = [&](const float4 &q) { return k == 0 ? q.x : k == 1 ? q.y : k == 2 ? q.z : q.w; };
+            const float2 a1 = make_float2(pick(qa), A[i1]);
+            float2 v = vsub(a1, pa);
+            pa = a1;
+            if (PREC == P_MIXED) {
+              const float2 x1 = make_float2(pick(qx), X[i1]);
+              v = vadd(v, vsub(x1, px));
+              px = x1;
+            }
+            return vmul(v, rd);
+          };
+        };
+        float2 *ox = su + lane * SUP + K * warp, *oy = sv + (K * segY) * TX + colY;
+        auto emit = [&](int q, float2 S, float2 D) {
+          ox[q] = make_float2(S.x, D.x);
+          oy[q * TX] = make_float2(S.y, D.y);
+        };
+        // the sweeps that give the one-sided derivatives themselves
+        auto emit_pm = [&](int q, float2 dm, float2 dp) { emit(q, vadd(dp, dm), vsub(dp, dm)); };
+        // arc length: the near-linear form first; segments that do not qualify take the full form, swept again by
+        // the warp where at least kWarpSegs fail (coarse grids, the rounding noise of FP32), else entered in a
+        // list whose nodes all threads of the CTA share (a kink crosses few segments of a tile, and the CTA
+        // would wait for their warps).  Both evaluate the same operations, so a node's derivatives depend only
+        // on the data of its 8-node segment, whose position on the grid is the same for both tile widths --
+        // not on the order in which tiles or instances are processed, nor on history: a single solve, a
+        // batch, a server round and a resumed checkpoint agree.
+        if constexpr (W == W_ARCLEN) {
+          // FP32 stores phi itself: its rounding over dx is what the derivatives carry anyway
+          float2 size = make_float2(0.0f, 0.0f);
+          if (PREC == P_F32) {
+            size = make_float2(fmaxf(fabsf(A[ix + 4]), fabsf(A[ix + K + 3])) * d.rdx,
+                               fmaxf(fabsf(A[iy + 3 * SW]), fabsf(A[iy + (K + 2) * SW])) * d.rdy);
+          }
+          // segments of rows or columns beyond the grid (ragged tiles) do not count
+          if (ty0 + lane >= ny || tx0 + K * warp >= nx) size.x = INFINITY;
+          if (tx0 + colY >= nx || ty0 + K * segY >= ny) size.y = INFINITY;
+          const int near = sweep_stream_near<K, float2>(
+              make_vat(), rd, make_float2(fmaf(d.dx, d.dx, eps), fmaf(d.dy, d.dy, eps)), size, emit);
+          if (__any_sync(0xffffffffu, near != 3)) {
+            const bool fx = !(near & 1), fy = !(near & 2);
+            if (__popc(__ballot_sync(0xffffffffu, fx)) + __popc(__ballot_sync(0xffffffffu, fy)) >= kWarpSegs) {
+              SweepConsts<float2> sc;
+              sc.eps4 = make_float2(4.0f * eps * d.rdx * d.rdx, 4.0f * eps * d.rdy * d.rdy);
+              sc.h2 = make_float2(0.5f * d.dx, 0.5f * d.dy);
+              sc.h3 = make_float2(d.dx * (1.0f / 3.0f), d.dy * (1.0f / 3.0f));
+              sc.mh6 = make_float2(d.dx * (-1.0f / 6.0f), d.dy * (-1.0f / 6.0f));
+              // -0, unknown to the assembler: it fuses a packed multiply (or one with a constant zero added) with
+              // a packed add that is its only reader, as at the first and the last position, and the scalar
+              // sweep of the list, where it does not, would differ in the last bit
+              const float2 nz = vsplat(-(float)(p.stage >> 8), rd);
+              auto v_at = make_vat();
+              sweep_stream<K, float2>([&](int m) { return vfma(v_at(m), rd, nz); }, sc,
+                                      [&](int q, float2 dm, float2 dp) {
+                                        const float2 S = vadd(dp, dm), D = vsub(dp, dm);
+                                        if (fx) ox[q] = make_float2(S.x, D.x);
+                                        if (fy) oy[q * TX] = make_float2(S.y, D.y);
+                                      });
+            } else {
+              // entry: line (row or column), segment along it, direction
+              if (fx) s_list[atomicAdd(&s_nlist, 1)] = (unsigned short)((lane * 8 + warp) * 2);
+              if (fy) s_list[atomicAdd(&s_nlist, 1)] = (unsigned short)((colY * 8 + segY) * 2 + 1);
+            }
           }
         } else {
-          const float xn = fmaf((float)gi, d.dx, d.xlo), yn = fmaf((float)gj, d.dy, d.ylo);
-          float ax, ay;
-          hsel.alpha(u.x, u.y, sy, dy, xn, yn, ax, ay);
-          const float aX = local_alpha ? ax : fax, aY = local_alpha ? ay : fay;
-          L = fmaf(aX * 0.5f, u.y, fmaf(aY * 0.5f, dy, -hsel.value(u.x, sy, xn, yn)));
-          if (inside) {
-            // L depends on all four one-sided derivatives: L * 0 is NaN exactly when L is not finite
-            nfin = fmaf(L, 0.0f, nfin);
-            amx = fmaxf(amx, ax);
-            // (with a runtime Hamiltonian the fold below does not copy amx, so amy is always kept)
-            if (!HS::kSameAlpha || !HamSel<H>::kSameAlpha) amy = fmaxf(amy, ay);
-          }
+          sweep_stream_jp<K, float2>(make_vat(), make_float2(eps, eps), emit_pm);
         }
-        if (ST == 0 || !inside) continue;
-        const int sidx = (y + 3) * SW + colY + 4;
-        const size_t g = rbase + (size_t)(gj + GY) * p.pitch + gi + GX;
-        if (PREC == P_MIXED) {
-          // phi^n = hi + lo (A, B) and the stage states phi_1 = hi + e_1, phi_2 = hi + e_2, where the
-          // increment arrays e_k = lo + (phi_k - phi^n) carry the low part (C = e_{k-1}):
-          //   e_1 = lo + dt L,  e_2 = 3/4 lo + 1/4 (e_1 + dt L),  phi^{n+1} = hi + lo + 2/3 (e_2 + dt L - lo)
-          // (Step 5's combinations with phi_k - phi^n = e_k - lo)
-          if (ST == 3) {
-            const float dd = (2.0f / 3.0f) * (fmaf(dtf, L, C[sidx]) - B[sidx]);
-            float h, l;
-            df_add(A[sidx], B[sidx], dd, h, l);
-            float *oh = reinterpret_cast<float *>(p.mix_hi[i_cur ^ 1]);
-            float *ol = reinterpret_cast<float *>(p.mix_lo[i_cur ^ 1]);
-            if (EDGE) {
-              store_node<float, 2>(oh + rbase, p.pitch, nx, ny, d.bc, gi, gj, h);
-              store_node<float, 2>(ol + rbase, p.pitch, nx, ny, d.bc, gi, gj, l);
-            } else {
-              oh[g] = h;
-              ol[g] = l;
+      }
+      __syncthreads();
+      if (W == W_ARCLEN && s_nlist > 0) {
+        for (int i = tid; i < s_nlist * K; i += NT) {
+          const int e = s_list[i / K], q = i % K, along_y = e & 1, line = e >> 4, at = ((e >> 1) & 7) * K + q;
+          const int step = along_y ? SW : 1, i0 = along_y ? at * SW + line + 4 : (line + 3) * SW + at + 1;
+          const float rdl = along_y ? d.rdy : d.rdx, dl = along_y ? d.dy : d.dx;
+          SweepConsts<float> sc;
+          sc.eps4 = 4.0f * eps * rdl * rdl;
+          sc.h2 = 0.5f * dl;
+          sc.h3 = dl * (1.0f / 3.0f);
+          sc.mh6 = dl * (-1.0f / 6.0f);
+          sweep_stream<1, float>(
+              [&](int m) {
+                const int j = i0 + m * step;
+                float v = vsub(A[j + step], A[j]);
+                if (PREC == P_MIXED) v = vadd(v, vsub(X[j + step], X[j]));
+                return vmul(vmul(v, rdl), rdl);
+              },
+              sc, [&](int, float dm, float dp) {
+                (along_y ? sv[at * TX + line] : su[line * SUP + at]) = make_float2(vadd(dp, dm), vsub(dp, dm));
+              });
+        }
+        __syncthreads();
+        if (tid == 0) s_nlist = 0;   // the next entries are made after the next tile's first barrier
+      }
+
+      // ---- 2. nodes (colY, K*segY + q): Lax-Friedrichs Hamiltonian, RK combination, store; one
+      // unrolled loop per stage and per edge/interior tile, so that no node tests either
+      float *out = reinterpret_cast<float *>(solo ? prm.outs[stage - 1] : p.out0);
+      auto finish = [&](auto stage_c, auto edge_c, auto hsel) {
+        using HS = decltype(hsel);
+        constexpr int ST = decltype(stage_c)::value;
+        constexpr bool EDGE = decltype(edge_c)::value;
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+          const int y = K * segY + q;
+          const float2 w = sv[y * TX + colY];    // (Sy, Dy)
+          const float sy = w.x, dy = w.y;
+          const int gi = tx0 + colY, gj = ty0 + y;
+          const bool inside = !EDGE || (gi < nx && gj < ny);
+          const float2 u = su[y * SUP + colY];   // (Sx, Dx)
+          float L;   // -H + alpha_x/2 Dx + alpha_y/2 Dy
+          if constexpr (HS::kGridFold) {
+            const float s = u.x + sy, e = fabsf(u.y) + fabsf(dy);
+            L = fmaf(faxh, u.y, fmaf(fayh, dy, -hsel.value(u.x, sy, 0.0f, 0.0f)));
+            if (inside) {
+              nfin = fmaf(L, 0.0f, nfin);
+              amx = fmaxf(amx, s + e);
+              amy = fmaxf(amy, e - s);
             }
           } else {
-            const float dd = (ST == 1) ? fmaf(dtf, L, B[sidx]) : fmaf(0.75f, B[sidx], 0.25f * fmaf(dtf, L, C[sidx]));
-            float *o = reinterpret_cast<float *>(p.out0);
-            if (EDGE) store_node<float, 2>(o + rbase, p.pitch, nx, ny, d.bc, gi, gj, dd);
-            else o[g] = dd;
+            const float xn = fmaf((float)gi, d.dx, d.xlo), yn = fmaf((float)gj, d.dy, d.ylo);
+            float ax, ay;
+            hsel.alpha(u.x, u.y, sy, dy, xn, yn, ax, ay);
+            const float aX = local_alpha ? ax : fax, aY = local_alpha ? ay : fay;
+            L = fmaf(aX * 0.5f, u.y, fmaf(aY * 0.5f, dy, -hsel.value(u.x, sy, xn, yn)));
+            if (inside) {
+              // L depends on all four one-sided derivatives: L * 0 is NaN exactly when L is not finite
+              nfin = fmaf(L, 0.0f, nfin);
+              amx = fmaxf(amx, ax);
+              // (with a runtime Hamiltonian the fold below does not copy amx, so amy is always kept)
+              if (!HS::kSameAlpha || !HamSel<H>::kSameAlpha) amy = fmaxf(amy, ay);
+            }
+          }
+          if (ST == 0 || !inside) continue;
+          const int sidx = (y + 3) * SW + colY + 4;
+          const size_t g = rbase + (size_t)(gj + GY) * p.pitch + gi + GX;
+          if (PREC == P_MIXED) {
+            // phi^n = hi + lo (A, B) and the stage states phi_1 = hi + e_1, phi_2 = hi + e_2, where the
+            // increment arrays e_k = lo + (phi_k - phi^n) carry the low part (C = e_{k-1}):
+            //   e_1 = lo + dt L,  e_2 = 3/4 lo + 1/4 (e_1 + dt L),  phi^{n+1} = hi + lo + 2/3 (e_2 + dt L - lo)
+            // (Step 5's combinations with phi_k - phi^n = e_k - lo)
+            if (ST == 3) {
+              const float dd = (2.0f / 3.0f) * (fmaf(dtf, L, C[sidx]) - B[sidx]);
+              float h, l;
+              df_add(A[sidx], B[sidx], dd, h, l);
+              float *oh = reinterpret_cast<float *>(p.mix_hi[i_cur ^ 1]);
+              float *ol = reinterpret_cast<float *>(p.mix_lo[i_cur ^ 1]);
+              if (EDGE) {
+                store_node<float, 2>(oh + rbase, p.pitch, nx, ny, d.bc, gi, gj, h);
+                store_node<float, 2>(ol + rbase, p.pitch, nx, ny, d.bc, gi, gj, l);
+              } else {
+                oh[g] = h;
+                ol[g] = l;
+              }
+            } else {
+              const float dd = (ST == 1) ? fmaf(dtf, L, B[sidx]) : fmaf(0.75f, B[sidx], 0.25f * fmaf(dtf, L, C[sidx]));
+              float *o = out;
+              if (EDGE) store_node<float, 2>(o + rbase, p.pitch, nx, ny, d.bc, gi, gj, dd);
+              else o[g] = dd;
+            }
+          } else {
+            const float src = A[sidx];
+            float outv;
+            if (ST == 1) {
+              outv = fmaf(dtf, L, src);
+            } else if (ST == 2) {
+              outv = fmaf(0.75f, B[sidx], 0.25f * fmaf(dtf, L, src));
+            } else {
+              outv = fmaf(1.0f / 3.0f, B[sidx], (2.0f / 3.0f) * fmaf(dtf, L, src));
+            }
+            float *o = out;
+            if (EDGE) store_node<float, 2>(o + rbase, p.pitch, nx, ny, d.bc, gi, gj, outv);
+            else o[g] = outv;
+          }
+        }
+      };
+      // the Hamiltonian of the tile: the launch's, or with H_RUNTIME the instance's, chosen once per tile
+      auto finish_h = [&](auto stage_c, auto edge_c) {
+        if constexpr (H == H_RUNTIME) {
+          switch (d.ham) {
+            case H_BURGERS2D: finish(stage_c, edge_c, HamSel<H_BURGERS2D>{}); break;
+            case H_NEGCOS2D: finish(stage_c, edge_c, HamSel<H_NEGCOS2D>{}); break;
+            case H_SIN2D: finish(stage_c, edge_c, HamSel<H_SIN2D>{}); break;
+            default: finish(stage_c, edge_c, HamSel<H_EIKONAL2D>{}); break;
           }
         } else {
-          const float src = A[sidx];
-          float outv;
-          if (ST == 1) {
-            outv = fmaf(dtf, L, src);
-          } else if (ST == 2) {
-            outv = fmaf(0.75f, B[sidx], 0.25f * fmaf(dtf, L, src));
-          } else {
-            outv = fmaf(1.0f / 3.0f, B[sidx], (2.0f / 3.0f) * fmaf(dtf, L, src));
-          }
-          float *o = reinterpret_cast<float *>(p.out0);
-          if (EDGE) store_node<float, 2>(o + rbase, p.pitch, nx, ny, d.bc, gi, gj, outv);
-          else o[g] = outv;
+          finish(stage_c, edge_c, HamSel<H>{});
         }
+      };
+      auto finish_stage = [&](auto stage_c) {
+        if (edge) finish_h(stage_c, std::true_type{});
+        else finish_h(stage_c, std::false_type{});
+      };
+      switch (stage) {
+        case 0: finish_stage(std::integral_constant<int, 0>{}); break;
+        case 1: finish_stage(std::integral_constant<int, 1>{}); break;
+        case 2: finish_stage(std::integral_constant<int, 2>{}); break;
+        default: finish_stage(std::integral_constant<int, 3>{}); break;
       }
-    };
-    // the Hamiltonian of the tile: the launch's, or with H_RUNTIME the instance's, chosen once per tile
-    auto finish_h = [&](auto stage_c, auto edge_c) {
-      if constexpr (H == H_RUNTIME) {
-        switch (d.ham) {
-          case H_BURGERS2D: finish(stage_c, edge_c, HamSel<H_BURGERS2D>{}); break;
-          case H_NEGCOS2D: finish(stage_c, edge_c, HamSel<H_NEGCOS2D>{}); break;
-          case H_SIN2D: finish(stage_c, edge_c, HamSel<H_SIN2D>{}); break;
-          default: finish(stage_c, edge_c, HamSel<H_EIKONAL2D>{}); break;
-        }
-      } else {
-        finish(stage_c, edge_c, HamSel<H>{});
-      }
-    };
-    auto finish_stage = [&](auto stage_c) {
-      if (edge) finish_h(stage_c, std::true_type{});
-      else finish_h(stage_c, std::false_type{});
-    };
-    switch (p.stage) {
-      case 0: finish_stage(std::integral_constant<int, 0>{}); break;
-      case 1: finish_stage(std::integral_constant<int, 1>{}); break;
-      case 2: finish_stage(std::integral_constant<int, 2>{}); break;
-      default: finish_stage(std::integral_constant<int, 3>{}); break;
-    }
 
-    // ---- when the next tile of this CTA belongs to another instance (or there is none), fold the
-    // run's maximum of alpha into the instance's slot and count its tiles; close the instance's stage
-    ++run_tiles;
-    const bool more = next < ntiles;
-    if (more && !s_info[buf ^ 1].skip && s_info[buf ^ 1].inst == i_inst) {
-      // no barrier: su, raw[buf] and s_info[buf] are rewritten only after the next tile's first
-      // barrier, which every thread reaches after finishing this tile
-      continue;
-    }
-    if constexpr (GF) {
-      amx = fmaxf(fmaxf(fmaf(0.5f, amx, 1.0f), fmaf(0.5f, amy, -1.0f)), 0.0f);
-      amy = amx;
-    } else if (HamSel<H>::kSameAlpha) {
-      amy = amx;
-    }
+      // ---- when the next tile of this CTA belongs to another instance (or there is none), fold the
+      // run's maximum of alpha into the instance's slot and count its tiles; close the instance's stage
+      ++run_tiles;
+      const bool more = next < ntiles;
+      if (more && !s_info[buf ^ 1].skip && s_info[buf ^ 1].inst == i_inst) {
+        // no barrier: su, raw[buf] and s_info[buf] are rewritten only after the next tile's first
+        // barrier, which every thread reaches after finishing this tile
+        continue;
+      }
+      if constexpr (GF) {
+        amx = fmaxf(fmaxf(fmaf(0.5f, amx, 1.0f), fmaf(0.5f, amy, -1.0f)), 0.0f);
+        amy = amx;
+      } else if (HamSel<H>::kSameAlpha) {
+        amy = amx;
+      }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      amx = fmaxf(amx, __shfl_xor_sync(0xffffffffu, amx, o));
-      amy = fmaxf(amy, __shfl_xor_sync(0xffffffffu, amy, o));
+      for (int o = 16; o > 0; o >>= 1) {
+        amx = fmaxf(amx, __shfl_xor_sync(0xffffffffu, amx, o));
+        amy = fmaxf(amy, __shfl_xor_sync(0xffffffffu, amy, o));
+      }
+      const int anybad = __syncthreads_or(nfin != nfin ? 1 : 0);
+      if (lane == 0) {
+        s_red[0][warp] = amx;
+        s_red[1][warp] = amy;
+      }
+      __syncthreads();
+      if (tid == 0) {
+        for (int w = 1; w < NT / 32; ++w) {
+          amx = fmaxf(amx, s_red[0][w]);
+          amy = fmaxf(amy, s_red[1][w]);
+        }
+        DevState *st = d.st;
+        if (solo) {
+          // a NaN stands for a non-finite dH/dp anywhere (the largest bit pattern)
+          atomicMax(&prm.solo->alpha[stage - 1][0], double_to_bits(anybad ? (double)NAN : (double)amx));
+          atomicMax(&prm.solo->alpha[stage - 1][1], double_to_bits((double)amy));
+        } else {
+          if (anybad) atomicOr(&st->err, 1);
+          if (p.write_slot >= 0) {
+            atomicMax(&st->alpha_bits[p.write_slot][0], double_to_bits((double)amx));
+            atomicMax(&st->alpha_bits[p.write_slot][1], double_to_bits((double)amy));
+          }
+          __threadfence();
+          const unsigned int prev = atomicAdd(&st->counter, (unsigned int)run_tiles);
+          if (prev + (unsigned int)run_tiles == (unsigned int)d.ntiles) {
+            // every tile of this instance has finished this stage
+            __threadfence();
+            st->counter = 0;
+            if (p.zero_slot >= 0) {
+              st->alpha_bits[p.zero_slot][0] = 0ull;
+              st->alpha_bits[p.zero_slot][1] = 0ull;
+            }
+            if (p.stage == 1 && p.loop_mode != LOOP_STAGE) {
+              st->dt = s_info[buf].dt;
+              st->last = s_info[buf].last;
+            }
+            if (p.stage == 3) {
+              if (PREC == P_MIXED) st->cur = i_cur ^ 1;
+              if (p.loop_mode != LOOP_STAGE) {
+                const double tn = st->last ? st->t_final : st->t + st->dt;
+                st->t = tn;
+                st->steps += 1;
+                if (p.loop_mode == LOOP_STEP_TO && !(tn < st->t_final) && prm.done_count) atomicAdd(prm.done_count, 1);
+              }
+            }
+          }
+        }
+      }
+      amx = amy = A0;
+      nfin = 0.0f;
+      run_tiles = 0;
+      __syncthreads();  // raw[buf], su, s_info[buf] are free for the next tile
     }
-    const int anybad = __syncthreads_or(nfin != nfin ? 1 : 0);
-    if (lane == 0) {
-      s_red[0][warp] = amx;
-      s_red[1][warp] = amy;
-    }
+    if (!solo) break;
+    // ---- grid barrier: the stage's outputs (ordinary stores) before the next one's tile loads (async proxy)
+    fence_proxy_async_global();
     __syncthreads();
     if (tid == 0) {
-      for (int w = 1; w < NT / 32; ++w) {
-        amx = fmaxf(amx, s_red[0][w]);
-        amy = fmaxf(amy, s_red[1][w]);
-      }
-      DevState *st = d.st;
-      if (anybad) atomicOr(&st->err, 1);
-      if (p.write_slot >= 0) {
-        atomicMax(&st->alpha_bits[p.write_slot][0], double_to_bits((double)amx));
-        atomicMax(&st->alpha_bits[p.write_slot][1], double_to_bits((double)amy));
-      }
+      volatile SoloState *sh = prm.solo;
       __threadfence();
-      const unsigned int prev = atomicAdd(&st->counter, (unsigned int)run_tiles);
-      if (prev + (unsigned int)run_tiles == (unsigned int)d.ntiles) {
-        // every tile of this instance has finished this stage
-        __threadfence();
-        st->counter = 0;
-        if (p.zero_slot >= 0) {
-          st->alpha_bits[p.zero_slot][0] = 0ull;
-          st->alpha_bits[p.zero_slot][1] = 0ull;
-        }
-        if (p.stage == 1 && p.loop_mode != LOOP_STAGE) {
-          st->dt = s_info[buf].dt;
-          st->last = s_info[buf].last;
-        }
-        if (p.stage == 3) {
-          if (PREC == P_MIXED) st->cur = i_cur ^ 1;
-          if (p.loop_mode != LOOP_STAGE) {
-            const double tn = st->last ? st->t_final : st->t + st->dt;
-            st->t = tn;
-            st->steps += 1;
-            if (p.loop_mode == LOOP_STEP_TO && !(tn < st->t_final) && prm.done_count) atomicAdd(prm.done_count, 1);
-          }
-        }
+      const unsigned long long target = (unsigned long long)(run + 1) * gridDim.x;
+      unsigned long long seen = atomicAdd(&prm.solo->arrived, 1ull) + 1;
+      for (int spin = 0; seen < target && spin < kBarrierSpins; ++spin) seen = sh->arrived;
+      __threadfence();
+      fence_proxy_async_global();
+      s_lost = seen < target;
+      // the maxima of the stage just closed; the step's end
+      const double a0 = bits_to_double(sh->alpha[stage - 1][0]), a1 = bits_to_double(sh->alpha[stage - 1][1]);
+      const bool bad = a0 != a0;
+      if (stage == 3) {
+        for (int i = 0; i < 2; ++i) so.ends[0][i] = so.a[i];
+        so.ends[1][0] = bad ? 0.0 : a0;
+        so.ends[1][1] = a1;
+        so.t = so.last ? so.tf : so.t + so.dt;
+        so.cur ^= 1;
+        ++so.steps;
+      }
+      so.a[0] = a0;
+      so.a[1] = a1;
+      if (bad) so.err = 1;
+    }
+    __syncthreads();
+    if (s_lost) {   // a CTA never arrived
+      if (tid == 0) atomicOr(&prm.inst0.st->err, 2);
+      return;
+    }
+  }
+  if (solo && blockIdx.x == 0 && tid == 0) {
+    // the state as launches of single stages would leave it
+    DevState *st = prm.inst0.st;
+    if (so.err) st->err |= so.err;
+    st->dt = so.dt;
+    st->last = so.last;
+    if (so.steps > 0) {
+      st->t = so.t;
+      st->steps += so.steps;
+      if (PREC == P_MIXED) st->cur = so.cur;
+      st->alpha_bits[0][0] = st->alpha_bits[0][1] = 0ull;
+      for (int i = 0; i < 2; ++i) {
+        st->alpha_bits[1][i] = double_to_bits(so.ends[0][i]);
+        st->alpha_bits[2][i] = double_to_bits(so.ends[1][i]);
       }
     }
-    amx = amy = A0;
-    nfin = 0.0f;
-    run_tiles = 0;
-    __syncthreads();  // raw[buf], su, s_info[buf] are free for the next tile
   }
 }
 
