@@ -22,12 +22,8 @@ __device__ __forceinline__ T ghost_value(int g, int n, int bc, Get get) {
     if (w < 0) w += n;
     return get(w);
   }
-  if (g < 0) {
-    const T m = T(-g);
-    return (T(1) + m) * get(0) - m * get(1);
-  }
-  const T m = T(g - (n - 1));
-  return (T(1) + m) * get(n - 1) - m * get(n - 2);
+  if (g < 0) return extrapolate<T>(-g, get(0), get(1));
+  return extrapolate<T>(g - (n - 1), get(n - 1), get(n - 2));
 }
 
 // One thread per (line, ghost position): rows first (x ghosts), then columns.

@@ -114,4 +114,12 @@ int launch_pack(const void *padded, int prec_elem /*0 f64, 1 f32*/, void *dst, i
 int launch_unpack(const void *src, int src_dtype, void *padded, int prec_elem, int nx, int ny, int pitch,
                   int dim, void *stream);
 
+#ifdef __CUDACC__
+// Ghost value m nodes beyond the end of a line whose last two values are a (at the end) and b.
+template <typename T>
+__device__ __forceinline__ T extrapolate(int m, T a, T b) {
+  return (T(1) + T(m)) * a - T(m) * b;
+}
+#endif
+
 }  // namespace alw

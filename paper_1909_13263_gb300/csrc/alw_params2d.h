@@ -44,8 +44,11 @@ struct Stage2DParams {
   const int *tiles;         // batch: work list, entry = instance * 65536 + tile of that instance
   int *done_count;          // batch: incremented when an instance reaches its t_final (may be null)
   InstDesc inst0;
-  // Whole RK3 steps of the single instance in one cooperative launch (nsteps > 0; lagged or fixed alpha,
-  // periodic): the stage, its maps, output and slots follow from the loop and a grid barrier separates the
+  // the stage extrapolates its output's ghosts itself (linear extrapolation, wide tiles; grids whose last tile
+  // column and row are at least two nodes wide, so that a line's last two nodes lie in one tile)
+  int ghosts;
+  // Whole RK3 steps of the single instance in one cooperative launch (nsteps > 0; lagged or fixed alpha, periodic
+  // or `ghosts`): the stage, its maps, output and slots follow from the loop and a grid barrier separates the
   // stages.  Zero at launch.
   int nsteps;
   void *outs[3];

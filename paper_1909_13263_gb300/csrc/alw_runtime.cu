@@ -144,7 +144,8 @@ struct alw_solver {
   cudaGraphExec_t g_adv = nullptr;
   bool has_phi = false;
   bool line64 = false;      // 1D FP64 grid that fits one cluster: many steps per launch
-  bool multi2d = false;     // periodic 2D float grid: several steps per cooperative launch
+  bool multi2d = false;     // 2D float grid: several steps per cooperative launch
+  bool ghosts2d = false;    // the 2D float kernel extrapolates the ghosts (see Stage2DParams)
   SoloState *solo = nullptr;  // what their CTAs share
   bool use2d = false;       // persistent TMA kernel (2D float variants)
   int shape64 = 0;          // FP64 2D: tile shape (kShape64)
@@ -180,7 +181,7 @@ int kernel_prec(int precision) {
   return precision == ALW_PREC_FP64 ? P_F64 : precision == ALW_PREC_FP32 ? P_F32 : P_MIXED;
 }
 
-// Periodic 2D float grids without a reduction pass before the stage run several steps per cooperative launch, so
+// 2D float grids without a reduction pass or ghost launch between stages run several steps per cooperative launch, so
 // many that a launch takes a millisecond or two.  The grid barrier between two stages costs less than a kernel's
 // end and the next one's start, at every size; measured (GB300, us per RK3 step of Example 3, a launch per stage
 // -> cooperative): 96^2 35 -> 26, 400^2 28.7 -> 18.5, 1024^2 43.1 -> 33.2, 2048^2 90.4 -> 83.3, 4096^2 279.9 ->
@@ -219,6 +220,7 @@ int launch_stage(const alw_solver *s, const StageParams &p, int nsteps = 0) {
     d.lx = s->lx;
     d.ly = s->ly;
     d.st = s->st;
+    q.ghosts = s->ghosts2d && p.stage != 0;
     if (nsteps > 0) {
       q.nsteps = nsteps;
       q.solo = s->solo;
@@ -343,7 +345,7 @@ constexpr int kLineSteps = 512;  // RK3 steps per launch of the 1D FP64 cluster 
 
 // Enqueue one RK3 step (with the reduction passes and ghost fills the mode needs).
 alw_status enqueue_step(alw_solver *s, int loop_mode) {
-  const bool linx = s->grid.bc == ALW_BC_LINEXTRAP;
+  const bool linx = s->grid.bc == ALW_BC_LINEXTRAP && !s->ghosts2d;
   for (int stage = 1; stage <= 3; ++stage) {
     const bool pre = (s->alpha_mode == ALW_ALPHA_GLOBAL_EXACT) || (s->alpha_mode == ALW_ALPHA_LOCAL_EXACT && stage == 1);
     if (pre) {
@@ -545,7 +547,8 @@ alw_status alw_create(const alw_grid *grid, const alw_hamiltonian *ham, const al
   s->elem = s->prec == P_F64 ? 8 : 4;
   s->use2d = s->dim == 2 && s->prec != P_F64;
   s->line64 = s->dim == 1 && s->prec == P_F64 && s->nx <= kLine64Max && !exact_mode(s->alpha_mode);
-  s->multi2d = s->use2d && !exact_mode(s->alpha_mode) && per;
+  s->ghosts2d = s->use2d && !per && s->nx % kTile2DX != 1 && s->ny % kTile2DY != 1;
+  s->multi2d = s->use2d && !exact_mode(s->alpha_mode) && (per || s->ghosts2d);
   s->arr_bytes = (size_t)s->pitch * s->rows * s->elem;
 
   auto cleanup = [&](alw_status st) {
@@ -749,7 +752,7 @@ alw_status alw_run_stage(alw_solver *s, int32_t stage, double dt) {
   StageParams p = make_params(s, stage, stage, LOOP_STAGE);
   p.dt_value = dt;
   ALW_LAUNCH(launch_stage(s, p));
-  if (s->grid.bc == ALW_BC_LINEXTRAP) ALW_LAUNCH(launch_ghosts(ghost_params(s, stage), s->stream));
+  if (s->grid.bc == ALW_BC_LINEXTRAP && !s->ghosts2d) ALW_LAUNCH(launch_ghosts(ghost_params(s, stage), s->stream));
   return ALW_OK;
 }
 

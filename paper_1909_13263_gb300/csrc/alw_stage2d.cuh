@@ -699,6 +699,44 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
         default: finish_stage(std::integral_constant<int, 3>{}); break;
       }
 
+      // ---- extrapolated boundary: the ghosts of the lines that end in this tile, from the two values just stored
+      // at their ends (as separate launches after the stage, they took a third of a step at 1024^2: 57.9 us against
+      // 37.1)
+      if constexpr (TX == kTile2DX && H != H_RUNTIME) {
+        if (prm.ghosts && edge) {
+          __syncthreads();
+          const int x0 = d.tx0, y0 = d.ty0, w = min(TX, d.nx - x0), h = min(TY, d.ny - y0);
+          auto hi = reinterpret_cast<float *>(p.mix_hi[d.cur ^ 1]), lo = reinterpret_cast<float *>(p.mix_lo[d.cur ^ 1]);
+          for (int c = warp; c < 12; c += NT / 32) {
+            const int side = c / 3, m = c % 3 + 1;   // left, right, lower, upper; nodes beyond the end
+            const bool ends = side == 0 ? x0 == 0 : side == 1 ? x0 + w == d.nx : side == 2 ? y0 == 0 : y0 + h == d.ny;
+            if (!ends) continue;
+            const int n = side < 2 ? h : w, dir = (side & 1) ? -1 : 1;   // inwards
+            const int sstep = dir * (side < 2 ? 1 : SW);
+            const long long gstep = dir * (side < 2 ? 1ll : (long long)p.pitch);
+            for (int i = lane; i < n; i += 32) {
+              const int x = side < 2 ? (side == 0 ? 0 : w - 1) : i, y = side < 2 ? i : (side == 2 ? 0 : h - 1);
+              const int s = (y + 3) * SW + x + 4;
+              const long long g = (long long)(d.row_off + y0 + y + GY) * p.pitch + x0 + x + GX;
+              if (PREC != P_MIXED) {
+                out[g - m * gstep] = extrapolate<float>(m, out[g], out[g + gstep]);
+              } else if (stage == 3) {
+                const double v = extrapolate<double>(m, (double)hi[g] + (double)lo[g],
+                                                     (double)hi[g + gstep] + (double)lo[g + gstep]);
+                const float vh = (float)v;
+                hi[g - m * gstep] = vh;
+                lo[g - m * gstep] = (float)(v - (double)vh);
+              } else {
+                // so that hi + increment is the extrapolated stage state (see ghosts_incr)
+                const double v = extrapolate<double>(m, (double)A[s] + (double)out[g],
+                                                     (double)A[s + sstep] + (double)out[g + gstep]);
+                out[g - m * gstep] = (float)(v - (double)A[s - m * sstep]);
+              }
+            }
+          }
+        }
+      }
+
       // ---- when the next tile of this CTA belongs to another instance (or there is none), fold the
       // run's maximum of alpha into the instance's slot and count its tiles; close the instance's stage
       ++run_tiles;

@@ -1,12 +1,13 @@
 """2D float solves whose RK3 steps run several to a launch, against the same steps made of single stages.
 
 Both run the same arithmetic on the same tiles, so every result is bitwise the same: the field, the grid
-maxima and the time.
+maxima and the time.  The ghosts that the stages extrapolate are checked through the oracle's stages, with the
+bound of one float stage (test_gpu_parity.py), restarted at every step from the kernel's own field.
 """
 import numpy as np
 import pytest
 
-from gpucase import Case
+from gpucase import Case, oracle_stages, rel_err
 from paper_1909_13263_gb300 import native
 
 pytestmark = pytest.mark.gpu
@@ -22,8 +23,9 @@ def _lib():
     yield
 
 
-def _case(shape, precision="mixed", weights="arclength", alpha_mode="global_lagged", ham="burgers2d"):
-    return Case(2, *shape, ham, precision=precision, weights=weights, alpha_mode=alpha_mode,
+def _case(shape, precision="mixed", weights="arclength", alpha_mode="global_lagged", ham="burgers2d",
+          bc="periodic"):
+    return Case(2, *shape, ham, bc=bc, precision=precision, weights=weights, alpha_mode=alpha_mode,
                 alpha_fixed=(2.5, 2.0) if alpha_mode == "fixed" else (0.0, 0.0), lo=-2.0, hi=2.0)
 
 
@@ -64,7 +66,8 @@ def _same(s, ref):
 
 @pytest.mark.parametrize("shape", SHAPES, ids=str)
 @pytest.mark.parametrize("kind", [dict(), dict(precision="fp32"), dict(weights="jp"), dict(alpha_mode="local_lagged"),
-                                  dict(alpha_mode="fixed"), dict(ham="eikonal2d", precision="fp32")], ids=str)
+                                  dict(alpha_mode="fixed"), dict(ham="eikonal2d", precision="fp32"),
+                                  dict(bc="linextrap"), dict(bc="linextrap", precision="fp32")], ids=str)
 def test_steps_of_one_launch_equal_single_stages(shape, kind):
     case = _case(shape, **kind)
     phi0 = _phi0(case)
@@ -94,3 +97,24 @@ def test_nonfinite_ends_the_launch_and_is_reported():
         s.advance(3)
         s.sync()
         assert s.get_state().steps == 3
+
+
+# the last tile two nodes wide and high (the narrowest that extrapolates in the stage), one node (separate ghost
+# launches), whole tiles, the smallest grid, more tiles than CTAs
+@pytest.mark.parametrize("precision", ["mixed", "fp32"])
+@pytest.mark.parametrize("shape", [(66, 34), (65, 34), (66, 33), (128, 64), (2, 2), (1500, 901)], ids=str)
+def test_extrapolated_ghosts_match_oracle(shape, precision):
+    case = _case(shape, precision=precision, alpha_mode="fixed", ham="sin2d", bc="linextrap")
+    case.alpha_fixed = (1.0, 1.0)
+    dt = 0.6 / (1.0 / case.dx + 1.0 / case.dy)
+    phi = case.field(seed=6)
+    with case.solver() as s:
+        s.set_phi0(phi)
+        errs = []
+        for _ in range(3):
+            ref = oracle_stages(case, phi, dt)
+            for stage in (1, 2, 3):
+                s.run_stage(stage, dt)
+                phi = s.get_stage_phi(stage) if stage < 3 else s.get_phi()
+                errs.append(rel_err(phi, ref[stage - 1]))
+    assert max(errs) <= 64 * 2.0**-24, errs
