@@ -359,14 +359,16 @@ __device__ __forceinline__ void sweep_stream_jp(LoadV v_at, V eps, Emit emit) {
     T[m] = vsub(dd[m], dd[m - 1]);
     T3[m] = vmul(T[m], c13);
   };
+  // indicators (13 (x - y)^2 + 3 a^2 + eps)^2 of the pair (x, y) = (s_m, s_{m+1}), a = x - 3 y, x + y, 3 x - y, from
+  // r = sqrt(3) s: the factor 3 is in the squares, and what all three share is formed once (13 packed operations
+  // against 19; Example 3, 4096^2 MIXED: 314 against 323 us per RK3 step)
+  V r[K + 5];
+  auto jp_r = [&](int m) { r[m] = vmul(vsplat(1.7320508075688772f, eps), s[m]); };
   auto jp_pair = [&](int m) {
-    const V x = s[m], y = s[m + 1];
-    const V d = vsub(x, y);
-    const V d13 = vmul(vsplat(13.0f, x), vmul(d, d));
-    const V a = vfma(vsplat(-3.0f, x), y, x), b = vadd(x, y), cc = vsub(vmul(vsplat(3.0f, x), x), y);
-    const V three = vsplat(3.0f, x);
-    const V ea = vadd(vfma(vmul(three, a), a, d13), eps), eb = vadd(vfma(vmul(three, b), b, d13), eps);
-    const V ec = vadd(vfma(vmul(three, cc), cc, d13), eps);
+    const V x = r[m], y = r[m + 1], d = vsub(x, y), m3 = vsplat(-3.0f, x);
+    const V e = vfma(vmul(vsplat(13.0f / 3.0f, x), d), d, eps);
+    const V a = vfma(m3, y, x), b = vadd(x, y), cc = vfma(m3, x, y);
+    const V ea = vfma(a, a, e), eb = vfma(b, b, e), ec = vfma(cc, cc, e);
     qX[m] = vmul(ea, ea);
     qY[m] = vmul(eb, eb);
     qZ[m] = vmul(ec, ec);
@@ -378,6 +380,8 @@ __device__ __forceinline__ void sweep_stream_jp(LoadV v_at, V eps, Emit emit) {
   for (int m = 1; m <= 5; ++m) pos_s(m);
 #pragma unroll
   for (int m = 2; m <= 4; ++m) pos_T(m);
+#pragma unroll
+  for (int m = 1; m <= 5; ++m) jp_r(m);
 #pragma unroll
   for (int m = 1; m <= 4; ++m) jp_pair(m);
 
@@ -396,6 +400,7 @@ __device__ __forceinline__ void sweep_stream_jp(LoadV v_at, V eps, Emit emit) {
       v[p + 6] = v_at(p + 6);
       pos_s(p + 6);
       pos_T(p + 5);
+      jp_r(p + 6);
       jp_pair(p + 5);
     }
   }
