@@ -25,7 +25,7 @@
 // The central parts are formed from d_m = s_{m+1} - s_m (s_m = v_m - v_{m-1}): for the node between
 // v_2 and v_3 of its window, c + T_b/12 = (v_2 + v_3)/2 - d_2/6 and c - T_b/12 = (v_2 + v_3)/2 - d_3/6,
 // and T_m = d_m - d_{m-1}; the widths d_m / dx are those of the arc-length intervals.  The arc-length
-// sweeps take their input as u = v / dx (the differences pass scales by 1/dx^2), so that the second
+// sweeps take their input as u = v / dx (the loads scale by 1/dx^2), so that the second
 // differences D2_m = u_m - u_{m-1} and the widths W_m = D2_{m+1} - D2_m = d_m / dx come without a
 // multiply; dx enters once, in the constants dx/2, dx/3, -dx/6 of the central parts and of T_a/3, T_b/2.
 // The Jiang-Peng sweep needs no D2 and keeps v.
@@ -192,7 +192,8 @@ __device__ __forceinline__ V q_interval_v(V nh, V rh, FValV<V> fa, FValV<V> fb, 
 }
 
 // Reciprocal of -nh from that of a width w that nh differs from by rounding only (one Newton step, for one special
-// function instruction per lane less: Example 3 on 8192^2, FP32, 1662 against 1689 us per RK3 step; where w vanishes against the ends the caller's trapezoid branch discards it).
+// function instruction per lane less: Example 3 on 8192^2, FP32, 1662 against 1689 us per RK3 step; where w
+// vanishes against the ends the caller's trapezoid branch discards it).
 template <class V>
 __device__ __forceinline__ V rcp_near(V nh, V rw) { return vfma(rw, vfma(nh, rw, vsplat(1.0f, nh)), rw); }
 
@@ -217,12 +218,12 @@ template <class V> struct SweepConsts {
 // den = A0 + 6 A1 + 3 A2 and num = A0 T_a / 3 + A2 T_b / 2 on either side (ta = T_a / 3, tb = T_b / 2 of
 // that side).  Each side's correction num / den is returned as a pair (num, r) with correction = num * r:
 // r = -1 / den on the "-" side (whose correction is subtracted) and 1 / den on the "+" side, so that the
-// caller adds num * r to the central part with one fused multiply-add.  CHECKED: on lanes whose
+// caller adds num * r to the central part with one fused multiply-add.  On lanes whose
 // denominator leaves the safe float range (or is NaN), num = the correction from side_corr_wide and
-// r = -1 or 1.  MINUS / PLUS select the sides wanted.  (The sweeps with the range check form each
-// side on its own -- sharing the products there measured slower, the rare out-of-line fallback
-// making the shared values live across its call -- and the short-interval sweep forms both.)
-template <bool CHECKED, bool MINUS, bool PLUS, class V>
+// r = -1 or 1.  MINUS / PLUS select the sides wanted.  (The sweeps form each side on its own:
+// sharing the products measured slower, the rare out-of-line fallback making the shared values live across
+// its call.)
+template <bool MINUS, bool PLUS, class V>
 __device__ __forceinline__ void group_corr_v(V g0, V g1, V g2, V ta_m, V tb_m, V ta_p, V tb_p, V &num_m, V &r_m,
                                              V &num_p, V &r_p) {
   using LN = Lanes<V>;
@@ -237,10 +238,10 @@ __device__ __forceinline__ void group_corr_v(V g0, V g1, V g2, V ta_m, V tb_m, V
 #pragma unroll
     for (int i = 0; i < LN::n; ++i) {
       const float dn = LN::get(den, i);
-      if (CHECKED) ok = ok && (dn < 1e30f);
+      ok = ok && (dn < 1e30f);
       LN::at(rd, i) = sfu_rcp(neg ? -dn : dn);
     }
-    if (CHECKED && !ok) {
+    if (!ok) {
 #pragma unroll
       for (int i = 0; i < LN::n; ++i) {
         const float dn = LN::get(den, i);
@@ -259,8 +260,7 @@ __device__ __forceinline__ void group_corr_v(V g0, V g1, V g2, V ta_m, V tb_m, V
 }
 
 // The extrapolated interval ends R_m = 2 D2_m - D2_{m-1} and L_m = 2 D2_m - D2_{m+1}, formed as
-// D2_m plus or minus the neighbouring width W (the quantity the short-interval test inspects; one
-// operation each).
+// D2_m plus or minus the neighbouring width W (one operation each).
 template <class V>
 __device__ __forceinline__ V r_end(V d2m, V w_prev) { return vadd(d2m, w_prev); }
 template <class V>
@@ -332,9 +332,9 @@ __device__ __forceinline__ void sweep_stream(LoadV u_at, const SweepConsts<V> &c
 #pragma unroll
   for (int p = 0; p < K; ++p) {
     V nm, rm, np, rp, unused0, unused1;
-    group_corr_v<true, true, false>(qX[p + 2], qY[p + 2], qZ[p + 3], w.Ta[p + 2], w.Tb[p + 3], w.Ta[p + 2],
+    group_corr_v<true, false>(qX[p + 2], qY[p + 2], qZ[p + 3], w.Ta[p + 2], w.Tb[p + 3], w.Ta[p + 2],
                                     w.Tb[p + 3], nm, rm, unused0, unused1);
-    group_corr_v<true, false, true>(qX[p + 3], qY[p + 3], qZ[p + 4], w.Ta[p + 3], w.Tb[p + 4], w.Ta[p + 4],
+    group_corr_v<false, true>(qX[p + 3], qY[p + 3], qZ[p + 4], w.Ta[p + 3], w.Tb[p + 4], w.Ta[p + 4],
                                     w.Tb[p + 3], unused0, unused1, np, rp);
     w.emit_node(p, c, nm, rm, np, rp, emit);
     // advance the window by one position
@@ -403,9 +403,9 @@ __device__ __forceinline__ void sweep_stream_jp(LoadV v_at, V eps, Emit emit) {
     const V mid = vmul(c12, vadd(v[p + 2], v[p + 3]));
     const V tb2 = vmul(c12, T[p + 3]);
     V nm, rm, np, rp, unused0, unused1;
-    group_corr_v<true, true, false>(qX[p + 1], qY[p + 2], qZ[p + 3], T3[p + 2], tb2, T3[p + 2], tb2, nm, rm,
+    group_corr_v<true, false>(qX[p + 1], qY[p + 2], qZ[p + 3], T3[p + 2], tb2, T3[p + 2], tb2, nm, rm,
                                     unused0, unused1);
-    group_corr_v<true, false, true>(qX[p + 2], qY[p + 3], qZ[p + 4], T3[p + 4], tb2, T3[p + 4], tb2, unused0,
+    group_corr_v<false, true>(qX[p + 2], qY[p + 3], qZ[p + 4], T3[p + 4], tb2, T3[p + 4], tb2, unused0,
                                     unused1, np, rp);
     emit(p, vfma(nm, rm, vfma(dd[p + 2], cm16, mid)), vfma(np, rp, vfma(dd[p + 3], cm16, mid)));
     if (p + 1 < K) {
