@@ -41,14 +41,15 @@ MUFU_PER_SM_CLK = 16          # measured: rsqrt / lg2 / rcp.approx throughput pe
 FP32_LANES_PER_SM = 128
 
 # algorithmic work of one 2D node in one stage (arc-length weights, Burgers H):
-# per direction 3 F evaluations (rsqrt + lg2), 3 interval means (1 reciprocal each),
-# 2 weight sets (1 reciprocal each) -> 11 MUFU ops; FP32 flops ~107 per direction
+# per direction 3 F evaluations (sqrt + lg2), 3 interval means (1 reciprocal for the three),
+# 2 weight sets (1 reciprocal each) -> 9 MUFU ops; FP32 flops ~107 per direction
 # plus ~33 for alpha, H-hat and the RK combination; bytes: each array read or written once per stage
-# (MIXED arc length on smooth data runs the short-interval sweep: per direction 3 square roots and
-# 2 weight reciprocals, 5 MUFU ops; "mufu_full" is the count of the full sweep)
+# (near-linear segments, all of this workload's in MIXED, take one reciprocal per stencil that serves both
+# sides: 2 per node; "mufu_full" is the count of the full sweep: per direction 3 x 2 for F, one reciprocal for
+# the three intervals, 2 for the weights)
 ALGO = {
-    ("arclength", "mixed"): {"mufu": 10, "mufu_full": 22, "flops": 250, "bytes": (12, 16, 20)},
-    ("arclength", "fp32"): {"mufu": 22, "flops": 240, "bytes": (8, 12, 12)},
+    ("arclength", "mixed"): {"mufu": 2, "mufu_full": 18, "flops": 250, "bytes": (12, 16, 20)},
+    ("arclength", "fp32"): {"mufu": 18, "flops": 240, "bytes": (8, 12, 12)},
     ("jp", "mixed"): {"mufu": 4, "flops": 180, "bytes": (12, 16, 20)},
     ("jp", "fp32"): {"mufu": 4, "flops": 170, "bytes": (8, 12, 12)},
     ("arclength", "fp64"): {"mufu": 0, "flops": 250, "bytes": (16, 24, 24)},
@@ -167,6 +168,15 @@ def _traffic():
     if t.get("source_hash") != _kernel_source_hash():
         return None
     return t
+
+
+def _stage_launches(args) -> int:
+    """Launches of the stage kernel in the timed region: a cooperative launch runs up to 64 whole steps of a float
+    grid (4 on the largest, as the runtime's multi_steps); FP64 launches every stage."""
+    if args.precision == "fp64":
+        return 3 * args.steps
+    per_launch = min(64, max(4, (1 << 24) // (args.n * args.n)))
+    return -(-args.steps // per_launch)
 
 
 def cpu_oracle_rate(n: int, steps: int):
@@ -593,7 +603,7 @@ def bench_fp64(args, stream):
         ms = e0.elapsed_time(e1) / args.fp64_steps
     return {"workload": f"ex3_burgers2d_{n}sq", "value": n * n / (ms * 1e-3), "unit": UNIT, "ms_per_step": ms,
             "steps": args.fp64_steps, "bound": "fp64 pipe",
-            "fp64_pipe_note": "ncu: FP64 pipe 86 % busy on this kernel (profiles/stage_kernel_fp64_ex3_arclength_1024.md)"}
+            "fp64_pipe_note": "56 FP64 operations per node and stage; ncu at 2048^2: FP64 pipe 80 % busy"}
 
 
 def run_ours(args):
@@ -636,7 +646,7 @@ def run_ours(args):
         ms = ev0.elapsed_time(ev1)
         clocks = cs.summary()
         # per-stage device time of the stage kernel, each stage launched alone (events on the launching
-        # stream): a breakdown only -- the roofline uses the launches inside the timed graph replays
+        # stream): a breakdown only -- the roofline uses the timed region
         st = s.get_state()
         dt = 0.6 / (st.alpha[0] / dx + st.alpha[1] / dx)
         reps = 5
@@ -699,18 +709,18 @@ def run_ours(args):
     peaks, src = _peaks()
     algo = ALGO.get((args.weights, args.precision), ALGO[("arclength", "mixed")])
     pts = n * n
-    # the dominant kernel's average launch duration inside the timed region: a periodic grid's RK3 step
-    # graph holds exactly the three stage launches (no ghost or reduction kernels), so the per-launch
-    # average is the graph-timed step time / 3 (graph gaps included: achieved is, if anything, low)
+    # the dominant kernel's average time per stage inside the timed region: nothing but its stages runs there
+    # (whole RK3 steps per cooperative launch in the float precisions, a launch per stage in FP64), so it is
+    # the step time / 3 (grid barriers and launch gaps included: achieved is, if anything, low)
     launch_ms = ms / (3 * args.steps)
-    bytes_launch = sum(algo["bytes"]) * pts / 3.0       # algorithmic bytes of an average stage launch
+    bytes_launch = sum(algo["bytes"]) * pts / 3.0       # algorithmic bytes of an average stage
     hbm_achieved = bytes_launch / (launch_ms * 1e-3) / 1e9
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
     mufu_achieved = algo["mufu"] * pts / (launch_ms * 1e-3) / 1e9        # Gop/s
     mufu_peak = SM_COUNT * MUFU_PER_SM_CLK * SM_MAX_MHZ * 1e6 / 1e9
     traffic = _traffic()
     roof = {
-        "kernel": "stage2d_kernel (3 launches per RK3 step; per-launch average over the timed graph replays)",
+        "kernel": "stage2d_kernel (average per stage over the timed region, 3 stages per RK3 step)",
         "bound": "hbm",
         "unit": "GB/s",
         "achieved": hbm_achieved,
@@ -769,7 +779,7 @@ def run_ours(args):
         "roofline": roof,
         "cpu_baseline": cpu,
         "e2e": e2e,
-        "gpu_launches": 3 * args.steps,
+        "gpu_launches": _stage_launches(args),
         "clocks": clocks,
         "batched": batched,
         "serving": serving,
