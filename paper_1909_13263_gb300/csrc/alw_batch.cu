@@ -575,7 +575,11 @@ alw_status autotune(alw_batch *b) {
       best = cands[i].t;
     }
   }
-  best.steps_per_graph = total >= 4096 ? 2 : (total >= 512 ? 8 : 32);
+  // A replay costs a read-back (about 15 us); steps captured beyond the last one still cost their launches, and each
+  // captured step its share of the graph's instantiation.  Measured (GB300, us per run at 2 / 4 / 8 / 32 steps): 6
+  // grids up to 160^2 1172 / 1133 / 1170 / 1369, 10 up to 300^2 1632 / 1561 / 1638 / 1673, 48 up to 512^2 (1600
+  // tiles) 5952 / 5924 / 6052 / 6610.
+  best.steps_per_graph = total >= 4096 ? 2 : 4;
   best.grid_ctas = 0;  // occupancy cap
   b->tuning = best;
   b->grid_cap = cap_for(b);
