@@ -319,19 +319,22 @@ ALW_HD void stencil_q(df D1, df D2, df D3, df D4, df w1, df w2, df w3, df &S2, c
 }
 
 // Scales a stencil's q's by the power of two that brings the largest to about one, so that their products
-// stay in the float range; returns the largest (before scaling; NaN and infinity fail the caller's test).
-ALW_HD float scale_q(df &q0, df &q1, df &q2) {
-  const float qm = fmaxf(q0.h, fmaxf(q1.h, q2.h));
+// stay in the float range; false when one of them (before scaling) is out of range: above 1e37 (or infinite), or
+// below 1e-27, where the low parts of the pair arithmetic that formed it run out of exponents (a product's
+// remainder, 2^-48 of it, must stay above 2^-149).  Arc length never goes below 16; Jiang-Peng does when eps and
+// the differences are both tiny.  NaN fails the caller's tests of the denominators.
+ALW_HD bool scale_q(df &q0, df &q1, df &q2) {
+  const float qm = fmaxf(q0.h, fmaxf(q1.h, q2.h)), qn = fminf(q0.h, fminf(q1.h, q2.h));
   const float sc = asf_(0x7f000000u - (asu_(qm) & 0x7f800000u));
   q0 = {q0.h * sc, q0.l * sc};
   q1 = {q1.h * sc, q1.l * sc};
   q2 = {q2.h * sc, q2.l * sc};
-  return qm;
+  return qm < 1e37f && qn > 1e-27f;
 }
 
 // Both deviations of a stencil, "-" of its node and "+" of the node before (times 20); false: out of range.
 ALW_HD bool stencil_devs(df q0, df q1, df q2, df T2, df T3, df &minus, df &plus) {
-  const float qm = scale_q(q0, q1, q2);
+  const bool ok = scale_q(q0, q1, q2);
   const df U = mul_(q2, sub_(q1, q0)), V = mul_(q0, sub_(q1, q2)), A1 = mul_(q0, q2);
   const df base = add_(mulf_(A1, 10.0f), add_(U, V));
   const df U2 = {U.h + U.h, U.l + U.l}, V2 = {V.h + V.h, V.l + V.l};
@@ -340,7 +343,7 @@ ALW_HD bool stencil_devs(df q0, df q1, df q2, df T2, df T3, df &minus, df &plus)
   const df np = add_(mul_(sub_(mulf_(V, 6.0f), U2), T3), mul_(sub_(mulf_(U, 7.0f), V), T2));
   minus = mul_(nm, rcp_(denA));
   plus = mul_(np, rcp_(denB));
-  return qm < 1e37f && denA.h > 1e-30f && denB.h > 1e-30f;
+  return ok && denA.h > 1e-30f && denB.h > 1e-30f;
 }
 
 // Magnitude of phi from the upper word of |phi|, 0 outside the float range
@@ -469,7 +472,7 @@ ALW_NOINLINE double minus64_rare(const double *a, int step, const Sweep64 &c) {
   df S = {0.0f, 0.0f}, q0, q1, q2;
   if (W == W_ARCLEN) S = root_(D[2]);
   stencil_q<W>(D[1], D[2], D[3], D[4], w[1], w[2], w[3], S, c, q0, q1, q2);
-  const float qm = scale_q(q0, q1, q2);
+  const bool ok = scale_q(q0, q1, q2);
   const df Ta = sub_(w[2], w[1]), Tb = sub_(w[3], w[2]);
   // phi^- = (v_2 + v_3)/2 - d_2/6 - (w0 2 T_a + w2 T_b)/6, the w_k proportional to n_k
   const df n0 = mul_(q1, q2), n1 = mulf_(mul_(q0, q2), 6.0f), n2 = mulf_(mul_(q0, q1), 3.0f);
@@ -489,7 +492,7 @@ ALW_NOINLINE double minus64_rare(const double *a, int step, const Sweep64 &c) {
     x = mul_(n1, nTb);
     y = mul_(n0, add_(Ta2, nTb));
   }
-  if (!(qm < 1e37f && r.h < 1e30f && (fabsf(x.h) + fabsf(y.h)) * r.h * c.t2phi <= (W == W_ARCLEN ? 2.0f : 1.0f) * phi_size(p)))
+  if (!(ok && r.h < 1e30f && (fabsf(x.h) + fabsf(y.h)) * r.h * c.t2phi <= (W == W_ARCLEN ? 2.0f : 1.0f) * phi_size(p)))
     return minus64_double<W>(a, step, c);
   const df z = mul_(add_(x, y), r);
   const double six = 1.0 / 6.0, cz = c.cdev * (20.0 / 6.0);

@@ -134,3 +134,23 @@ def test_line_solve_reports_nonfinite():
             s.step_to(1.0)
         assert e.value.status == native.ENONFINITE
         assert s.get_state().steps == 1
+
+
+# Jiang-Peng indicators far below one: q = (eps + 13 d^2 + 3 e^2)^2 reaches and passes the smallest float, down to
+# where only double holds it.  H is linear in the derivatives to first order (advection, sin(p + q)), so that phi
+# keeps the size of the data.
+@pytest.mark.parametrize("eps, size", [(1e-24, 1e-10), (1e-24, 1e-12), (1e-40, 1e-11), (1e-40, 5e-13), (1e-30, 3e-12),
+                                       (1e-18, 1e-9), (1e-300, 1e-20)])
+@pytest.mark.parametrize("dim, nx", [(1, 80), (1, 320), (1, 2000), (2, 80)])
+def test_small_jiang_peng_indicators_match_oracle(dim, nx, eps, size):
+    case = Case(dim, nx, 70 if dim == 2 else 1, "sin2d" if dim == 2 else "advect1d", weights="jp", eps=eps, lo=-2.0,
+                hi=2.0, alpha_mode="global_lagged" if dim == 2 else "local_lagged")
+    phi0 = size * _smooth(case)
+    assert max(_errors(case, phi0)) <= FP64_TOL
+    # the same step by the solver's own loop (1D: the kernel that runs whole steps)
+    a, _ = oracle.alpha_of(case.cfg(), phi0)
+    dt = 0.6 / (a[0] / case.dx + (a[1] / case.dy if dim == 2 else 0.0))
+    with case.solver() as s:
+        s.set_phi0(phi0)
+        s.advance(1)
+        assert rel_err(s.get_phi(), oracle_stages(case, phi0, dt)[2]) <= FP64_TOL
