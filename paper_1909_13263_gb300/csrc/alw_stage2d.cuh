@@ -40,15 +40,17 @@
 namespace alw {
 
 // Hamiltonians of the 2D examples in float (compile-time kind), from the sums and differences of a node's
-// one-sided derivatives, Sx = u^+ + u^-, Dx = u^+ - u^-, Sy = v^+ + v^-, Dy = v^+ - v^-: value is H at the mean
-// derivatives, alpha the maximum of |H_p| and |H_q| over the four corners.  u^-+ = (Sx -+ Dx)/2, so the corner
+// one-sided derivatives, Sx = u^+ + u^-, Dx = u^+ - u^-, Sy = v^+ + v^-, Dy = v^+ - v^-: value is kUnit H at the mean
+// derivatives (a power of two: the finish loop forms kUnit L and steps by dt / kUnit, both exactly, which saves
+// Burgers the multiplication by 1/2 of every node), alpha the maximum of |H_p| and |H_q| over the four corners.  u^-+ = (Sx -+ Dx)/2, so the corner
 // sums u + v are (Sx + Sy)/2 +- (Dx + Dy)/2 and +- (Dx - Dy)/2, and the largest and smallest |u| are
 // (|Sx| +- |Dx|)/2 in magnitude.
 template <int H> struct Ham2;
 template <> struct Ham2<H_BURGERS2D> {
   static constexpr bool kSameAlpha = true;
+  static constexpr float kUnit = 0.5f;
   __device__ __forceinline__ static float value(float su, float sv, float, float) {
-    const float z = fmaf(0.353553390593274f, su + sv, 0.707106781186548f);   // ((su + sv)/2 + 1) / sqrt 2
+    const float z = fmaf(0.25f, su + sv, 0.5f);   // half of p + q + 1
     return z * z;
   }
   // |H_p| = |H_q| = |u + v + 1|: at the largest or the smallest corner sum, (s +- e)/2
@@ -67,6 +69,7 @@ __device__ __forceinline__ float corner_max(float c, float dx, float dy, F f) {
 }
 template <> struct Ham2<H_NEGCOS2D> {
   static constexpr bool kSameAlpha = true;
+  static constexpr float kUnit = 1.0f;
   __device__ __forceinline__ static float value(float su, float sv, float, float) {
     return -sfu_cos(fmaf(0.5f, su + sv, 1.0f));
   }
@@ -77,6 +80,7 @@ template <> struct Ham2<H_NEGCOS2D> {
 };
 template <> struct Ham2<H_SIN2D> {
   static constexpr bool kSameAlpha = true;
+  static constexpr float kUnit = 1.0f;
   __device__ __forceinline__ static float value(float su, float sv, float, float) { return sfu_sin(0.5f * (su + sv)); }
   __device__ __forceinline__ static void alpha(float sx, float dx, float sy, float dy, float, float, float &ax,
                                                float &ay) {
@@ -85,6 +89,7 @@ template <> struct Ham2<H_SIN2D> {
 };
 template <> struct Ham2<H_EIKONAL2D> {
   static constexpr bool kSameAlpha = false;
+  static constexpr float kUnit = 1.0f;
   __device__ __forceinline__ static float value(float su, float sv, float, float) {
     const float p = 0.5f * su, q = 0.5f * sv, t = fmaf(p, p, fmaf(q, q, 1.0f));   // >= 1
     return t * sfu_rsqrt(t);
@@ -102,6 +107,7 @@ template <> struct Ham2<H_EIKONAL2D> {
 // Example 11 (optimal control): the only Hamiltonian that depends on the node position (x, y).
 template <> struct Ham2<H_OPTCTRL2D> {
   static constexpr bool kSameAlpha = false;
+  static constexpr float kUnit = 1.0f;
   __device__ __forceinline__ static float value(float su, float sv, float x, float y) {
     const float p = 0.5f * su, q = 0.5f * sv, sx = sfu_sin(x), cx = sfu_cos(x), sy = sfu_sin(y);
     // sin(y) p + (sin(x) + sign q) q - sin^2(y)/2 - (1 - cos x), with (sign q) q = |q|
@@ -126,6 +132,7 @@ constexpr int H_RUNTIME = -1;
 constexpr int H_BURGERS2D_GRID = -2;
 template <int H> struct HamSel {
   static constexpr bool kSameAlpha = Ham2<H>::kSameAlpha;
+  static constexpr float kUnit = Ham2<H>::kUnit;
   static constexpr bool kGridFold = false;
   __device__ __forceinline__ float value(float su, float sv, float x, float y) const {
     return Ham2<H>::value(su, sv, x, y);
@@ -460,7 +467,6 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
       const int nx = d.nx, ny = d.ny, tx0 = d.tx0, ty0 = d.ty0;
       const size_t rbase = (size_t)d.row_off * p.pitch;   // element offset of the instance's rows
       const float dtf = s_info[buf].dtf, fax = s_info[buf].fax, fay = s_info[buf].fay;
-      const float faxh = 0.5f * fax, fayh = 0.5f * fay;
       const float *A = raw + buf * NARR * ARR;
       const float *B = A + ARR;
       const float *C = A + 2 * ARR;
@@ -607,6 +613,8 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
         using HS = decltype(hsel);
         constexpr int ST = decltype(stage_c)::value;
         constexpr bool EDGE = decltype(edge_c)::value;
+        constexpr float U = HS::kUnit;
+        const float dtu = (1.0f / U) * dtf, faxh = (0.5f * U) * fax, fayh = (0.5f * U) * fay;
 #pragma unroll
         for (int q = 0; q < K; ++q) {
           const int y = K * segY + q;
@@ -615,7 +623,7 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
           const int gi = tx0 + colY, gj = ty0 + y;
           const bool inside = !EDGE || (gi < nx && gj < ny);
           const float2 u = su[y * SUP + colY];   // (Sx, Dx)
-          float L;   // -H + alpha_x/2 Dx + alpha_y/2 Dy
+          float L;   // U (-H + alpha_x/2 Dx + alpha_y/2 Dy)
           if constexpr (HS::kGridFold) {
             const float s = u.x + sy, e = fabsf(u.y) + fabsf(dy);
             L = fmaf(faxh, u.y, fmaf(fayh, dy, -hsel.value(u.x, sy, 0.0f, 0.0f)));
@@ -628,8 +636,8 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
             const float xn = fmaf((float)gi, d.dx, d.xlo), yn = fmaf((float)gj, d.dy, d.ylo);
             float ax, ay;
             hsel.alpha(u.x, u.y, sy, dy, xn, yn, ax, ay);
-            const float aX = local_alpha ? ax : fax, aY = local_alpha ? ay : fay;
-            L = fmaf(aX * 0.5f, u.y, fmaf(aY * 0.5f, dy, -hsel.value(u.x, sy, xn, yn)));
+            const float aX = local_alpha ? ax * (0.5f * U) : faxh, aY = local_alpha ? ay * (0.5f * U) : fayh;
+            L = fmaf(aX, u.y, fmaf(aY, dy, -hsel.value(u.x, sy, xn, yn)));
             if (inside) {
               // L depends on all four one-sided derivatives: L * 0 is NaN exactly when L is not finite
               nfin = fmaf(L, 0.0f, nfin);
@@ -647,7 +655,7 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
             //   e_1 = lo + dt L,  e_2 = 3/4 lo + 1/4 (e_1 + dt L),  phi^{n+1} = hi + lo + 2/3 (e_2 + dt L - lo)
             // (Step 5's combinations with phi_k - phi^n = e_k - lo)
             if (ST == 3) {
-              const float dd = (2.0f / 3.0f) * (fmaf(dtf, L, C[sidx]) - B[sidx]);
+              const float dd = (2.0f / 3.0f) * (fmaf(dtu, L, C[sidx]) - B[sidx]);
               float h, l;
               df_add(A[sidx], B[sidx], dd, h, l);
               float *oh = reinterpret_cast<float *>(p.mix_hi[i_cur ^ 1]);
@@ -660,7 +668,7 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
                 ol[g] = l;
               }
             } else {
-              const float dd = (ST == 1) ? fmaf(dtf, L, B[sidx]) : fmaf(0.75f, B[sidx], 0.25f * fmaf(dtf, L, C[sidx]));
+              const float dd = (ST == 1) ? fmaf(dtu, L, B[sidx]) : fmaf(0.75f, B[sidx], 0.25f * fmaf(dtu, L, C[sidx]));
               float *o = out;
               if (EDGE) store_node<float, 2>(o + rbase, p.pitch, nx, ny, d.bc, gi, gj, dd);
               else o[g] = dd;
@@ -669,11 +677,11 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
             const float src = A[sidx];
             float outv;
             if (ST == 1) {
-              outv = fmaf(dtf, L, src);
+              outv = fmaf(dtu, L, src);
             } else if (ST == 2) {
-              outv = fmaf(0.75f, B[sidx], 0.25f * fmaf(dtf, L, src));
+              outv = fmaf(0.75f, B[sidx], 0.25f * fmaf(dtu, L, src));
             } else {
-              outv = fmaf(1.0f / 3.0f, B[sidx], (2.0f / 3.0f) * fmaf(dtf, L, src));
+              outv = fmaf(1.0f / 3.0f, B[sidx], (2.0f / 3.0f) * fmaf(dtu, L, src));
             }
             float *o = out;
             if (EDGE) store_node<float, 2>(o + rbase, p.pitch, nx, ny, d.bc, gi, gj, outv);

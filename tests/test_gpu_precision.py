@@ -36,3 +36,25 @@ def test_mixed_l1_within_105_percent_of_fp64_where_discretisation_dominates(n):
 def test_mixed_beats_fp32_by_orders_of_magnitude_on_fine_grids():
     e64, emx, e32 = _solve(400, "fp64"), _solve(400, "mixed"), _solve(400, "fp32")
     assert emx < 2.0 * e64 and e32 > 20.0 * emx, (e64, emx, e32)
+
+
+# Where phi_x = phi_y = 0 Burgers' H is 1/2, and with a time step of 2^-6 every stage of Step 5 is exact in float:
+# the change over a step is -2^-7 to the last bit (up to the float 2/3 and 1/3 of stage 3, half a unit of the
+# increment or of phi).  A rounding bias of H, however small, shows here at full size and would grow with t.
+@pytest.mark.parametrize("precision", ["mixed", "fp32"])
+@pytest.mark.parametrize("alpha_mode", ["global_lagged", "local_lagged", "fixed"])
+def test_burgers_hamiltonian_is_unbiased_on_constants(precision, alpha_mode):
+    value, dt, steps = 0.25, 2.0**-6, 8
+    fixed = (1.0, 1.0) if alpha_mode == "fixed" else (0.0, 0.0)
+    with native.Solver(dim=2, nx=70, ny=40, xlo=-2.0, xhi=2.0, ylo=-2.0, yhi=2.0, ham="burgers2d", precision=precision,
+                       alpha_mode=alpha_mode, alpha_fixed=fixed) as s:
+        s.set_phi0(np.full((40, 70), value))
+        for _ in range(steps):
+            s.run_stage(1, dt)
+            if _ == 0:
+                np.testing.assert_array_equal(s.get_stage_phi(1), value - dt / 2)
+            s.run_stage(2, dt)
+            s.run_stage(3, dt)
+        err = np.abs(s.get_phi() - (value - steps * dt / 2)).max()
+    unit = dt / 2 if precision == "mixed" else value
+    assert err <= steps * unit * 2.0**-24
