@@ -635,7 +635,7 @@ alw_status alw_server_submit(alw_server *s, const alw_grid *grid, const alw_hami
   s->queue.push_back(r);
   s->stats.submitted++;
   *req_id = r->id;
-  s->cv.notify_one();
+  s->cv.notify_all();  // both threads wait on cv: waking only the compute thread would leave the request queued
   return ALW_OK;
 }
 

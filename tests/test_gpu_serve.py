@@ -94,3 +94,19 @@ def test_served_results_match_oracle():
         ref, _ = oracle_solve(inst, "arclength")
         err = float(np.max(np.abs(out - ref)))
         assert err <= MIXED_SOLVE_TOL, (inst, err)
+
+
+def test_idle_server_takes_a_single_request():
+    # nothing else to do on either thread: the one request has to wake the right one, and no later one helps
+    inst = inputs.batch_instances(1, 24, 64, seed=3)[0]
+    phi0, _ = inputs.instance_phi0(inst)
+    ref, steps = _single(inst)
+    for pause in (0.05, 0.2):
+        with native.Server(hbm_budget_bytes=1 << 28, max_slots=2, max_side=128) as srv:
+            for _ in range(3):
+                time.sleep(pause)
+                rid = srv.submit(nx=inst.n, ny=inst.n, xlo=-2.0, xhi=2.0, ylo=-2.0, yhi=2.0, ham=inst.ham, phi0=phi0,
+                                 t_final=inst.t_final)
+                done, info, out = srv.poll(rid, timeout=10.0)
+                assert done and info["status"] == 0 and info["steps"] == steps
+                np.testing.assert_array_equal(out, ref)
