@@ -536,8 +536,8 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
         // the warp where at least kWarpSegs fail (coarse grids, the rounding noise of FP32), else entered in a
         // list whose nodes all threads of the CTA share (a kink crosses few segments of a tile, and the CTA
         // would wait for their warps).  Both evaluate the same operations, so a node's derivatives depend only
-        // on the data of its 8-node segment, whose position on the grid is the same for both tile widths --
-        // not on the order in which tiles or instances are processed, nor on history: a single solve, a
+        // on the data of its 8-node segment and its ghosts, whose position on the grid is the same for both tile
+        // widths -- not on the order in which tiles or instances are processed, nor on history: a single solve, a
         // batch, a server round and a resumed checkpoint agree.
         if constexpr (W == W_ARCLEN) {
           // FP32 stores phi itself: its rounding over dx is what the derivatives carry anyway
@@ -546,11 +546,16 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
             size = make_float2(fmaxf(fabsf(A[ix + 4]), fabsf(A[ix + K + 3])) * d.rdx,
                                fmaxf(fabsf(A[iy + 3 * SW]), fabsf(A[iy + (K + 2) * SW])) * d.rdy);
           }
-          // segments of rows or columns beyond the grid (ragged tiles) do not count
-          if (ty0 + lane >= ny || tx0 + K * warp >= nx) size.x = INFINITY;
-          if (tx0 + colY >= nx || ty0 + K * segY >= ny) size.y = INFINITY;
-          const int near = sweep_stream_near<K, float2>(
-              make_vat(), rd, make_float2(fmaf(d.dx, d.dx, eps), fmaf(d.dy, d.dy, eps)), size, emit);
+          // segments of rows or columns beyond the grid (ragged tiles) do not count; segments that cross the grid's
+          // end are swept in full: beyond the three ghosts lies padding, which in the server's arena holds values
+          // of earlier requests, and the near test takes all of a segment's cells
+          const int endx = nx - tx0 - K * warp, endy = ny - ty0 - K * segY;   // nodes of the segment's line left
+          const bool outx = ty0 + lane >= ny || endx <= 0, outy = tx0 + colY >= nx || endy <= 0;
+          if (outx) size.x = INFINITY;
+          if (outy) size.y = INFINITY;
+          const int whole = (endx < K ? 0 : 1) | (endy < K ? 0 : 2), out = (outx ? 1 : 0) | (outy ? 2 : 0);
+          const int near = out | (whole & sweep_stream_near<K, float2>(make_vat(), rd,
+              make_float2(fmaf(d.dx, d.dx, eps), fmaf(d.dy, d.dy, eps)), size, emit));
           if (__any_sync(0xffffffffu, near != 3)) {
             const bool fx = !(near & 1), fy = !(near & 2);
             if (__popc(__ballot_sync(0xffffffffu, fx)) + __popc(__ballot_sync(0xffffffffu, fy)) >= kWarpSegs) {

@@ -110,3 +110,28 @@ def test_idle_server_takes_a_single_request():
                 done, info, out = srv.poll(rid, timeout=10.0)
                 assert done and info["status"] == 0 and info["steps"] == steps
                 np.testing.assert_array_equal(out, ref)
+
+
+# A slot's rows are reused.  The last 8-node segment of a ragged line reaches past the grid's ghosts into what an
+# earlier, larger request left there; here that continues the later request's data smoothly (and the later data do
+# not vanish at their edge, so that cleared padding would be a jump), which must not change a bit of its result.
+@pytest.mark.parametrize("precision", ["mixed", "fp32"])
+@pytest.mark.parametrize("n", [61, 59, 64])
+def test_result_does_not_depend_on_an_earlier_request(n, precision):
+    dx, big = 4.0 / n, 80
+
+    def data(m):
+        x = -2.0 + dx * np.arange(m)
+        return 0.3 + 0.01 * (np.sin(0.5 * np.pi * x)[None, :] + np.sin(0.5 * np.pi * x)[:, None])
+
+    kw = dict(nx=n, ny=n, xlo=-2.0, xhi=2.0, ylo=-2.0, yhi=2.0, ham="burgers2d")
+    first = dict(kw, nx=big, ny=big, xhi=-2.0 + big * dx, yhi=-2.0 + big * dx)
+    with native.Solver(dim=2, precision=precision, **kw) as s:
+        s.set_phi0(data(n))
+        s.step_to(0.2)
+        ref = s.get_phi()
+    with native.Server(hbm_budget_bytes=1 << 28, max_slots=1, max_side=128, precision=precision) as srv:
+        for job in (dict(first, phi0=data(big), t_final=0.0), dict(kw, phi0=data(n), t_final=0.2)):
+            done, info, out = srv.poll(srv.submit(**job), timeout=60.0)
+            assert done and info["status"] == 0
+    np.testing.assert_array_equal(out, ref)
