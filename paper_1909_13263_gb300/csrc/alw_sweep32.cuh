@@ -39,8 +39,9 @@
 //   lin^-+ = (v_2 + v_3)/2 -+ ... = (v_2 + v_3)/2 + W_1/30 - 3 W_2/20 - W_3/20  ("+": mirrored, from W_4),
 // one reciprocal and no square root per stencil for both sides.  sweep_stream_near evaluates this and bounds what
 // it leaves out: in units of D2 = dx^2-scaled differences (T, W the segment's largest) second-order terms
-// of the weights (0.04 T^3), of the indicators (0.01 T^3) and the interval widths' share of them
-// (0.01 T^2 W + 0.0025 T^2 W^2).  The segment qualifies when that is at most 2^-25 of its largest difference
+// of the weights and of the indicators (0.05 T^3) and the interval widths' share of them (0.0125 T^2 W + 0.0025
+// T^2 W^2); the largest omission over 3e6 random stencils is 0.94 of that sum (of 0.01 T^2 W it was 1.17).  The
+// segment qualifies when that is at most 2^-25 of its largest difference
 // (half a unit of the derivatives' own rounding), or, for a phi stored in float, 2^-25 of |phi| / dx (the
 // rounding of phi itself).  |y|/(y^2 + dx^2) <= 1/(2 dx), whence the bounds hold for any y.  Other
 // segments are swept with sweep_stream; the choice depends on the segment's own data only.
@@ -58,6 +59,10 @@
 namespace alw {
 
 constexpr float kNearTol = 1.0f / 33554432.0f;  // 2^-25
+// the bound of a near-linear stencil's omission: T^2 (kNearT T + kNearTW W + kNearTWW W^2)
+constexpr float kNearT = 0.05f;
+constexpr float kNearTW = 0.0125f;
+constexpr float kNearTWW = 0.0025f;
 
 // ---- lane-wise operations on float and float2 ------------------------------------------
 // Every add, subtract and multiply is rounded as written: the packed forms are PTX instructions
@@ -424,7 +429,7 @@ template <class V>
 __device__ __forceinline__ int near_mask(V tm, V wm, V vm, V rdx, V size) {
   using LN = Lanes<V>;
   const V t = vmul(tm, rdx), w = vfma(wm, rdx, t);        // |W| <= the nearest sample + |T|
-  const V f = vfma(w, vfma(vsplat(0.0025f, t), w, vsplat(0.01f, t)), vmul(vsplat(0.05f, t), t));
+  const V f = vfma(w, vfma(vsplat(kNearTWW, t), w, vsplat(kNearTW, t)), vmul(vsplat(kNearT, t), t));
   const V en = vmul(vmul(tm, t), f);                      // units of v
   int near = 0;
 #pragma unroll
@@ -477,7 +482,7 @@ __device__ __forceinline__ int sweep_stream_near(LoadV v_at, V rdx, V e1, V size
   };
   // Both early tests count too, so that stopping at them changes no segment's outcome.  A phi stored in float
   // whose rounding is n = 2^-25 |phi| / dx^2 gives T of 12 to 17 n (measured), which misses the bound where
-  // 0.05 T^3 > n.
+  // kNearT T^3 > n.
   int begun = 0;
 #pragma unroll
   for (int i = 0; i < LN::n; ++i) {
