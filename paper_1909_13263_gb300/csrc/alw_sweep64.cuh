@@ -11,14 +11,18 @@
 // V = A2 - A1 and den = A0 + 6 A1 + 3 A2.  The linear part, which carries the accuracy of phi, stays
 // in double; the deviation is a weight error (w - d) times third differences T, and is formed in unevaluated
 // float pairs (df).  Its error, measured against 128-bit arithmetic on smooth, kinked and noisy data, is at
-// most 2^-46.5 |T|.  A node takes this form when that stays below a quarter of the last place of phi itself:
-// |T| 2^8 (in units of phi) at most |phi|, so that 2^-46.5 |T| cfl < 2^-55 |phi|.
+// most 2^-46.5 |T|.  A node takes this form when |T| 2^10 (in units of phi) is at most |phi|, so that its error over
+// a stage, 2^-46.5 |T| cfl, is below 2^-57 |phi|, a sixteenth of phi's last place.
 // Next to a kink T is as large as the jump and that fails, but there the weights of the stencils that
 // cross the kink nearly vanish.  The node is then expanded about its dominant candidate k,
 //   phi^- = phi^{-,k} + sum over the others of w_l (phi^{-,l} - phi^{-,k}),
 // with the candidate in double and the sum in pairs, if the terms of the sum meet the bound (their sizes
-// times 2^7, Jiang-Peng 2^8, at most |phi|: they enter with 1/6).
+// times 2^9, Jiang-Peng 2^10, at most |phi|).
 // Nodes that fail both (noise, data the grid does not resolve) are computed in double.
+// The error of the one-sided derivatives against extended precision, as a share of that with double-precision
+// indicators (1000 lines of 40 to 1040 nodes each with sharp kinks, rounded corners or steep slopes): rms 0.68-0.79,
+// largest 0.19-0.86.  With 2^8, 2^7 and 2^8 for the three limits the largest were up to 4 times as large as the double
+// sweep's at kinks, and up to 14 times on finer grids.
 //
 // Arc-length indicators: with sigma = sqrt(1 + a^2) + sqrt(1 + b^2), h = b - a and t = h / sigma (= tanh of
 // half the difference of asinh b and asinh a), the mean of sqrt(1 + u^2) over [a, b], (F(b) - F(a)) / (2 h)
@@ -32,10 +36,9 @@
 // fit the instruction cache (2.1 stall cycles per issue waiting for instructions).
 //
 // Measured (GB300, RK3 steps of Example 3, against the sweep with double indicators): 2048^2 18.6 -> 1.53 ms per
-// step, 400^2 1570 -> 99 us; Example 10 on 1024^2 (kinks, double sine and cosine) 8.4 -> 0.81 ms.  The error of
-// the one-sided derivatives against 128-bit arithmetic is the double sweep's or smaller (cosine data, dx = 0.1
-// to 5e-4: 0.9-1.3e-16 rms against 0.9-1.8e-16).  What bounds it: the FP64 pipe, 56 operations per node (28
-// cycles of an SM; 80 % busy at 2048^2).
+// step, 400^2 1570 -> 99 us; Example 10 on 1024^2 (kinks, double sine and cosine) 8.4 -> 0.81 ms.  On smooth
+// data (cosine, dx = 0.1 to 5e-4) the error of the one-sided derivatives is 0.9-1.3e-16 rms against 0.9-1.8e-16.
+// What bounds it: the FP64 pipe, 56 operations per node (28 cycles of an SM; 80 % busy at 2048^2).
 #pragma once
 #include <string.h>
 
@@ -179,7 +182,7 @@ struct Sweep64 {
   double rdx, dx, eps_d;  // for the double form and the dominant-candidate form
   df scale;               // second differences of phi to the units of the indicators
   df eps;                 // arc length: 4 eps / dx^2; Jiang-Peng: eps
-  float t2phi;            // 2^8 T in units of phi
+  float t2phi;            // 2^10 T in units of phi
 };
 
 template <int W>
@@ -204,7 +207,7 @@ inline Sweep64 make_sweep64(double dx, double eps) {
   c.cdev = arc ? dx / 20.0 : 0.05 / 32.0;
   c.scale = pair(arc ? rdx * rdx : 32.0 * rdx);
   c.eps = pair(arc ? 4.0 * eps * rdx * rdx : 1024.0 * eps);
-  c.t2phi = (float)(256.0 * (arc ? dx * dx : dx / 32.0));
+  c.t2phi = (float)(1024.0 * (arc ? dx * dx : dx / 32.0));
   return c;
 }
 
@@ -408,9 +411,9 @@ template <int W>
 ALW_HD double minus64_double(const double *a, int step, const Sweep64 &c) {
   double v[5], s[5];
 #pragma unroll
-  for (int k = 0; k < 5; ++k) v[k] = (a[(k + 1) * step] - a[k * step]) * c.rdx;
+  for (int k = 0; k < 5; ++k) v[k] = a[(k + 1) * step] - a[k * step];
 #pragma unroll
-  for (int k = 1; k < 5; ++k) s[k] = v[k] - v[k - 1];
+  for (int k = 1; k < 5; ++k) s[k] = (v[k] - v[k - 1]) * c.rdx;   // (scaled last: the differences are nearly exact)
   const double d2 = s[3] - s[2], Ta = (s[1] + s[3]) - 2.0 * s[2], Tb = (s[2] + s[4]) - 2.0 * s[3];
   double q[3];
   if (W == W_ARCLEN) {
@@ -446,7 +449,7 @@ ALW_HD double minus64_double(const double *a, int step, const Sweep64 &c) {
     w2 = a2 / sum;
   }
   // (v_2 + v_3)/2 - d_2/6 - (w0 2 T_a + w2 T_b)/6
-  return fma(-1.0 / 6.0, fma(w0, 2.0 * Ta, fma(w2, Tb, d2)), 0.5 * (v[2] + v[3]));
+  return fma(-1.0 / 6.0, fma(w0, 2.0 * Ta, fma(w2, Tb, d2)), c.c0 * (v[2] + v[3]));
 }
 
 // phi^- of the node at cell a + 3 step where the linear expansion does not serve: about the dominant candidate,
