@@ -38,6 +38,16 @@ template <int PREC, int DIM, int SHAPE = 0> struct Shape {
   static constexpr int MINB = (PREC == P_F64 && DIM == 2) ? kShape64[SHAPE].warps * 32 / NT : 1;
   static constexpr int SW = TX + 8;                 // smem row: GX halo on each side
   static constexpr int SH = (DIM == 2) ? TY + 6 : 1;
+  // FP64 2D: sides that did not qualify from which a tile's threads sweep their own segments in double instead of
+  // sharing a list of sides: a sixth of all.  The list costs twice the FP64 operations (nothing is shared between the
+  // sides of a stencil) after a pair form in vain; a thread's sweep idles where few of its warp's segments have such
+  // nodes.  Microseconds per RK3 step, always the list / from a half / from a sixth; with double indicators throughout:
+  //   Example 3, noise on all nodes    2048^2 57290 / 16580 / 16580; 15040     512^2 3820 / 1155 / 1155; 1149
+  //   noise on 3 % of them                    23250 / 19290 / 15840; 24740           2060 / 1410 / 1150; 1605
+  //   noise on 1 %                            10760 / 10720 / 12240; 24970           1250 / 1110 / 1080; 1755
+  //   shocks of a long run              256^2 666 / 364 / 242; 581    Example 10, 1024^2 1128 / 918 / 860; 8330
+  //   Jiang-Peng, noise on all         2048^2 17210 / 5660 / 5660; 5000
+  static constexpr int kDense = 2 * DIM * TX * TY / 6;
   static constexpr int NARR = (PREC == P_MIXED) ? 3 : 1;
   static constexpr size_t smem_bytes() {
     return (size_t)NARR * SH * SW * sizeof(typename Types<PREC>::S) +
@@ -200,7 +210,8 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SHAPE>::NT, Shape<PREC, DIM, 
     // finishing a node needs (registers)
     double2 *su = reinterpret_cast<double2 *>(s_u), *sv = su + (DIM - 1) * TY * TX;
     unsigned short *s_rare = reinterpret_cast<unsigned short *>(su + DIM * TY * TX);
-    {
+    unsigned mine;   // the thread's segment: nodes that did not qualify
+    auto segment = [&](auto use) {
       constexpr int SEGS = TX / K;
       const int dir = (DIM == 2 && tid >= Sh::NSEG) ? 1 : 0, seg = tid - dir * Sh::NSEG;
       const int x = dir == 0 ? (seg % SEGS) * K : seg % TX, y = dir == 0 ? seg / SEGS : (seg / TX) * K;
@@ -209,20 +220,30 @@ __global__ void __launch_bounds__(Shape<PREC, DIM, SHAPE>::NT, Shape<PREC, DIM, 
       // nodes of the segment that lie inside the grid
       const int left = dir == 0 ? p.nx - tx0 - x : p.ny - ty0 - y;
       const bool inside = dir == 0 ? (DIM == 1 || ty0 + y < p.ny) : tx0 + x < p.nx;
+      use(a, step, dir, node0, ostep, !inside || left <= 0 ? -1 : (left < K ? left : K));
+    };
+    segment([&](const S *a, int step, int dir, int node0, int ostep, int nv) {
       double2 *o = (dir == 0 ? su : sv) + node0;
-      unsigned rare = sweep64<WEIGHTS>(a, step, sw.c[dir], !inside || left <= 0 ? -1 : (left < K ? left : K),
-                                       [&](int q, double dm, double dp) { o[q * ostep] = make_double2(dm, dp); });
+      mine = sweep64<WEIGHTS>(a, step, sw.c[dir], nv,
+                              [&](int q, double dm, double dp) { o[q * ostep] = make_double2(dm, dp); });
       // nodes that did not qualify: both sides of each into the CTA's list
-      while (rare) {
-        const int q = __ffs(rare) - 1;
-        rare &= rare - 1;
-        const int at = atomicAdd(&s_nrare, 2);
+      for (unsigned rare = mine; rare; rare &= rare - 1) {
+        const int q = __ffs(rare) - 1, at = atomicAdd(&s_nrare, 2);
         s_rare[at] = (unsigned short)(((dir * TY * TX + node0 + q * ostep) << 1));
         s_rare[at + 1] = (unsigned short)(s_rare[at] | 1);
       }
-    }
+    });
     __syncthreads();
-    if (s_nrare > 0) {
+    if (DIM == 2 && s_nrare >= Sh::kDense) {
+      // ... many (noise, data that the grid does not resolve): each thread its segment's, in double
+      if (mine) {
+        segment([&](const S *a, int step, int dir, int node0, int ostep, int) {
+          sweep64_double<WEIGHTS>(a, step, sw.c[dir], mine, reinterpret_cast<double *>((dir == 0 ? su : sv) + node0),
+                                  ostep);
+        });
+      }
+      __syncthreads();
+    } else if (s_nrare > 0) {
       // ... which all threads share: the kinks of a tile touch few threads' segments
       for (int i = tid; i < s_nrare; i += NT) {
         const int e = s_rare[i] >> 1, dir = e / (TY * TX), n = e % (TY * TX), x = n % TX, y = n / TX;

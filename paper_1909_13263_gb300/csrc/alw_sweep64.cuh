@@ -18,7 +18,8 @@
 //   phi^- = phi^{-,k} + sum over the others of w_l (phi^{-,l} - phi^{-,k}),
 // with the candidate in double and the sum in pairs, if the terms of the sum meet the bound (their sizes
 // times 2^9, Jiang-Peng 2^10, at most |phi|).
-// Nodes that fail both (noise, data the grid does not resolve) are computed in double.
+// Nodes that fail both (noise, data the grid does not resolve) are computed in double, side by side or, where a
+// tile holds many, segment by segment with each stencil's indicators shared by the two sides it serves.
 // The error of the one-sided derivatives against extended precision, as a share of that with double-precision
 // indicators (1000 lines of 40 to 1040 nodes each with sharp kinks, rounded corners or steep slopes): rms 0.68-0.79,
 // largest 0.19-0.86.  With 2^8, 2^7 and 2^8 for the three limits the largest were up to 4 times as large as the double
@@ -356,16 +357,18 @@ ALW_HD float phi_size(unsigned p) {
 
 // ---- the same in double, with FP64 operations saved where they can be: roots and reciprocals refine the
 // float approximation by Newton steps (7 and 4 operations), one logarithm per long interval only
+ALW_HD bool narrows_(double a) { return (hi_(a) & 0x7fffffffu) - 0x3a000000u < 0x47e00000u - 0x3a000000u; }
+ALW_HD float narrow_(double a) {  // towards zero, by bit patterns (the conversion instruction runs at the FP64 rate)
+  return asf_(shl3_(lo_(a), (hi_(a) & 0x7fffffffu) - 0x38000000u) | (hi_(a) & 0x80000000u));
+}
 ALW_HD double rcp64_(double a) {
-  const float f = rcp_((float)a);
-  if (!(fabsf(f) > 1e-37f && fabsf(f) < 1e37f)) return 1.0 / a;
-  double r = widen_(f);
-  r = fma(r, fma(-a, r, 1.0), r);
+  if (!narrows_(a)) return 1.0 / a;
+  const double f = widen_(rcp_(narrow_(a))), r = fma(f, fma(-a, f, 1.0), f);
   return fma(r, fma(-a, r, 1.0), r);
 }
 ALW_HD double sqrt64_(double a) {  // a >= 1
-  if (!(a < 1e37)) return sqrt(a);
-  const double y = widen_(rsq_((float)a));
+  if (!narrows_(a)) return sqrt(a);
+  const double y = widen_(rsq_(narrow_(a)));
   double g = a * y, h = 0.5 * y;
   const double r = fma(-g, h, 0.5);
   g = fma(g, r, g);
@@ -391,35 +394,33 @@ ALW_HD double log64_(double y) {  // y >= 1, as log_ (terms up to z^23)
   const double w = 2.0 * z;
   return fma((double)((int)k - 1023), 0.69314718055994530942, fma(w * z2, p, w));
 }
-ALW_HD double mean64_(double a, double sa, double b, double sb) {  // G (see the header comment)
-  const double h = b - a, sg = sa + sb, r = rcp64_(sg), t = h * r, x = t * t;
-  if (fabs(t) <= 0.25) {
+// G: by its series (see the header comment) or, for long intervals, as (F(b) - F(a)) / (2 h) with asinh b - asinh a =
+// ln((sigma + h)/(sigma - h)).  That cancels nothing that counts: (sigma - |h|)(sigma + |h|) >= 4 and |h| > sigma / 4,
+// so the rounding of sigma - |h| moves G by at most 2^-51 of itself.
+ALW_HD double mean64_(double a, double sa, double b, double sb) {
+  const double h = b - a, sg = sa + sb, d = fabs(h);
+  if (d <= 0.25 * sg) {
+    const double r = rcp64_(sg), t = h * r, x = t * t;
     double p = 26.0 / 27.0;
 #pragma unroll
     for (int k = 12; k >= 1; --k) p = fma(p, x, 2.0 * k / (2.0 * k + 1.0));
     return fma(-x * p, r, 0.5 * sg);
   }
-  const bool up = h > 0.0;
-  const double lo = up ? a : b, slo = up ? sa : sb, hi = up ? b : a, shi = up ? sb : sa, d = fabs(h), m = a + b;
-  const double t1 = lo >= 0.0 ? slo + lo : rcp64_(slo - lo), t2 = hi <= 0.0 ? shi - hi : rcp64_(shi + hi);
-  const double l = log64_((sg + d) * rcp64_(t1 + t2));
-  return 0.5 * fma(0.5, fma(m * m, r, sg), l * rcp64_(d));
+  const bool up = h > 0.0;   // the same bits whichever end comes first
+  const double n = fma(up ? b : a, up ? sb : sa, -((up ? a : b) * (up ? sa : sb)));
+  double w = sg - d;
+  if ((int)hi_(w) <= 0) w = hilo_(hi_(sg) - (53u << 20), 0u);   // rounded away (ends beyond 1e7: l does not count)
+  const double i = rcp64_(w * d), l = log64_((sg + d) * (d * i));
+  return 0.5 * (n + l) * (w * i);
 }
 
-// phi^- of the node at cell a + 3 step in double
+// Squared indicators of a stencil in double from its second differences s (over dx).  S2 = sqrt(1 + (s2 / dx)^2) on
+// entry, of s3 on return (arc length).
 template <int W>
-ALW_HD double minus64_double(const double *a, int step, const Sweep64 &c) {
-  double v[5], s[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) v[k] = a[(k + 1) * step] - a[k * step];
-#pragma unroll
-  for (int k = 1; k < 5; ++k) s[k] = (v[k] - v[k - 1]) * c.rdx;   // (scaled last: the differences are nearly exact)
-  const double d2 = s[3] - s[2], Ta = (s[1] + s[3]) - 2.0 * s[2], Tb = (s[2] + s[4]) - 2.0 * s[3];
-  double q[3];
+ALW_HD void stencil64_(double s1, double s2, double s3, double s4, double &S2, const Sweep64 &c, double (&q)[3]) {
   if (W == W_ARCLEN) {
-    const double u1 = s[1] * c.rdx, u2 = s[2] * c.rdx, u3 = s[3] * c.rdx, u4 = s[4] * c.rdx;
-    const double R = 2.0 * u2 - u1, L = 2.0 * u3 - u4;
-    const double S2 = sqrt64_(fma(u2, u2, 1.0)), S3 = sqrt64_(fma(u3, u3, 1.0));
+    const double u1 = s1 * c.rdx, u2 = s2 * c.rdx, u3 = s3 * c.rdx, u4 = s4 * c.rdx;
+    const double R = 2.0 * u2 - u1, L = 2.0 * u3 - u4, S3 = sqrt64_(fma(u3, u3, 1.0));
     q[0] = mean64_(u2, S2, R, sqrt64_(fma(R, R, 1.0)));
     q[1] = mean64_(u2, S2, u3, S3);
     q[2] = mean64_(L, sqrt64_(fma(L, L, 1.0)), u3, S3);
@@ -428,7 +429,9 @@ ALW_HD double minus64_double(const double *a, int step, const Sweep64 &c) {
       const double b = c.dx * q[k], e = fma(b, b, c.eps_d);
       q[k] = e * e;
     }
+    S2 = S3;
   } else {
+    const double s[5] = {0.0, s1, s2, s3, s4};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const double x = s[k + 1], y = s[k + 2], d = x - y, z = k == 0 ? x - 3.0 * y : (k == 1 ? x + y : 3.0 * x - y);
@@ -436,20 +439,69 @@ ALW_HD double minus64_double(const double *a, int step, const Sweep64 &c) {
       q[k] = e * e;
     }
   }
-  // omega_0, omega_2 in product form, or by quotients when the products leave the range
-  const double n0 = 0.1 * (q[1] * q[2]), n2 = 0.3 * (q[0] * q[1]), den = fma(0.6, q[0] * q[2], n0 + n2);
+}
+
+// w_0 2 T_a + w_2 T_b + d_2 of a side, so that phi^- = (v_2 + v_3)/2 - (...)/6; the "+" side is minus the mirrored
+// one.  omega_0, omega_2 in product form, or by quotients when the products leave the range.
+ALW_HD double side64_(double q0, double q1, double q2, double s1, double s2, double s3, double s4) {
+  const double d2 = s3 - s2, Ta = (s1 + s3) - 2.0 * s2, Tb = (s2 + s4) - 2.0 * s3;
+  const double n0 = 0.1 * (q1 * q2), n2 = 0.3 * (q0 * q1), den = fma(0.6, q0 * q2, n0 + n2);
   double w0, w2;
   if (den > 1e-290 && den < 1e290) {
     const double r = den > 1e-35 && den < 1e35 ? rcp64_(den) : 1.0 / den;
     w0 = n0 * r;
     w2 = n2 * r;
   } else {
-    const double a0 = 0.1 / q[0], a1 = 0.6 / q[1], a2 = 0.3 / q[2], sum = a0 + a1 + a2;
+    const double a0 = 0.1 / q0, a1 = 0.6 / q1, a2 = 0.3 / q2, sum = a0 + a1 + a2;
     w0 = a0 / sum;
     w2 = a2 / sum;
   }
-  // (v_2 + v_3)/2 - d_2/6 - (w0 2 T_a + w2 T_b)/6
-  return fma(-1.0 / 6.0, fma(w0, 2.0 * Ta, fma(w2, Tb, d2)), c.c0 * (v[2] + v[3]));
+  return fma(w0, 2.0 * Ta, fma(w2, Tb, d2));
+}
+
+ALW_HD double root64_(double s, const Sweep64 &c) { return sqrt64_(fma(s * c.rdx, s * c.rdx, 1.0)); }
+
+// phi^- of the node at cell a + 3 step in double
+template <int W>
+ALW_HD double minus64_double(const double *a, int step, const Sweep64 &c) {
+  double v[5], s[5], q[3];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) v[k] = a[(k + 1) * step] - a[k * step];
+#pragma unroll
+  for (int k = 1; k < 5; ++k) s[k] = (v[k] - v[k - 1]) * c.rdx;   // (scaled last: the differences are nearly exact)
+  double S = W == W_ARCLEN ? root64_(s[2], c) : 0.0;
+  stencil64_<W>(s[1], s[2], s[3], s[4], S, c, q);
+  return fma(-1.0 / 6.0, side64_(q[0], q[1], q[2], s[1], s[2], s[3], s[4]), c.c0 * (v[2] + v[3]));
+}
+
+// Both sides of the nodes `rare` of a segment in double, the bits of minus64_double's: the "-" side of node j and the
+// "+" side of node j - 1 share stencil j's indicators.  (phi^-, phi^+) of node q go to o[2 q ostep], o[2 q ostep + 1].
+template <int W>
+ALW_NOINLINE void sweep64_double(const double *a, int step, const Sweep64 &c, unsigned rare, double *o, int ostep) {
+  int j = 0, last = 0;
+  while (!(rare >> j & 1u)) ++j;
+  while (rare >> last) ++last;
+  const double *p = a + j * step;
+  double x = p[4 * step], v1 = p[2 * step] - p[step], v2 = p[3 * step] - p[2 * step], v3 = x - p[3 * step];
+  double s1 = (v1 - (p[step] - p[0])) * c.rdx, s2 = (v2 - v1) * c.rdx, s3 = (v3 - v2) * c.rdx;
+  double S = W == W_ARCLEN ? root64_(s2, c) : 0.0;
+#pragma unroll 1
+  for (; j <= last; ++j) {
+    const double y = a[(j + 5) * step], v4 = y - x, s4 = (v4 - v3) * c.rdx;
+    double q[3];
+    stencil64_<W>(s1, s2, s3, s4, S, c, q);
+    if (rare >> j & 1u)
+      o[2 * j * ostep] = fma(-1.0 / 6.0, side64_(q[0], q[1], q[2], s1, s2, s3, s4), c.c0 * (v2 + v3));
+    if (j > 0 && (rare >> (j - 1) & 1u))
+      o[2 * (j - 1) * ostep + 1] = fma(1.0 / 6.0, side64_(q[2], q[1], q[0], s4, s3, s2, s1), c.c0 * (v1 + v2));
+    x = y;
+    v1 = v2;
+    v2 = v3;
+    v3 = v4;
+    s1 = s2;
+    s2 = s3;
+    s3 = s4;
+  }
 }
 
 // phi^- of the node at cell a + 3 step where the linear expansion does not serve: about the dominant candidate,

@@ -154,3 +154,18 @@ def test_small_jiang_peng_indicators_match_oracle(dim, nx, eps, size):
         s.set_phi0(phi0)
         s.advance(1)
         assert rel_err(s.get_phi(), oracle_stages(case, phi0, dt)[2]) <= FP64_TOL
+
+
+# Tiles in which many nodes do not qualify are swept in double segment by segment, others node by node.  Noise over
+# part of the grid gives both, next to tiles that qualify; grids as above, so that the tile shapes and the ragged
+# segments of each are met.
+@pytest.mark.parametrize("weights", ["arclength", "jp"])
+@pytest.mark.parametrize("nx, ny", [(31, 33), (64, 48), (161, 163), (1025, 130), (600, 611)])
+def test_tiles_of_noise_match_oracle(nx, ny, weights):
+    case = Case(2, nx, ny, "sin2d", weights=weights, lo=-2.0, hi=2.0)
+    phi0 = _smooth(case)
+    rough = case.field(seed=8)
+    phi0[: ny // 3, : nx // 2] += 0.1 * rough[: ny // 3, : nx // 2]
+    scattered = np.random.default_rng(9).random((ny - ny // 2, nx)) < 0.05
+    phi0[ny // 2:][scattered] += 0.1 * rough[ny // 2:][scattered]
+    assert max(_errors(case, phi0)) <= FP64_TOL
