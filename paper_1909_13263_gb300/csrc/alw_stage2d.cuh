@@ -549,11 +549,17 @@ __global__ void __launch_bounds__(Geo2D<TXv>::NT, Geo2D<TXv>::MINB)
           // segments of rows or columns beyond the grid (ragged tiles) do not count; segments that cross the grid's
           // end are swept in full: beyond the three ghosts lies padding, which in the server's arena holds values
           // of earlier requests, and the near test takes all of a segment's cells
-          const int endx = nx - tx0 - K * warp, endy = ny - ty0 - K * segY;   // nodes of the segment's line left
-          const bool outx = ty0 + lane >= ny || endx <= 0, outy = tx0 + colY >= nx || endy <= 0;
-          if (outx) size.x = INFINITY;
-          if (outy) size.y = INFINITY;
-          const int whole = (endx < K ? 0 : 1) | (endy < K ? 0 : 2), out = (outx ? 1 : 0) | (outy ? 2 : 0);
+          // (only border tiles have any; in MIXED the test costs more than what it saves -- 8192^2, us per RK3 step of
+          // Example 3 without / with it: FP32 1682 / 1652, MIXED 1013 / 1027)
+          int out = 0, whole = 3;
+          if (PREC == P_MIXED || edge) {
+            const int endx = nx - tx0 - K * warp, endy = ny - ty0 - K * segY;   // nodes of the segment's line left
+            const bool outx = ty0 + lane >= ny || endx <= 0, outy = tx0 + colY >= nx || endy <= 0;
+            if (outx) size.x = INFINITY;
+            if (outy) size.y = INFINITY;
+            whole = (endx < K ? 0 : 1) | (endy < K ? 0 : 2);
+            out = (outx ? 1 : 0) | (outy ? 2 : 0);
+          }
           const int near = out | (whole & sweep_stream_near<K, float2>(make_vat(), rd,
               make_float2(fmaf(d.dx, d.dx, eps), fmaf(d.dy, d.dy, eps)), size, emit));
           if (__any_sync(0xffffffffu, near != 3)) {
