@@ -321,6 +321,27 @@ alw_status build_graph(alw_batch *b, int nsteps, int ntiles) {
 
 alw_status prime_alpha(alw_batch *b) { return launch_groups(b, 0, LOOP_ADVANCE, 0.0); }
 
+// Graph replays before the next read-back: by the instances' last time steps, as many as it takes until half of the
+// uploaded tiles are done and the work list is compacted (or everything is), rounded down.
+int replays_ahead(const alw_batch *b, const std::vector<char> &live, int tiles_listed) {
+  std::vector<std::pair<double, int>> left;   // steps to go, tiles
+  long long tiles = 0;
+  for (size_t i = 0; i < live.size(); ++i) {
+    if (!live[i]) continue;
+    const DevState &s = b->h_state[i];
+    left.emplace_back(s.dt > 0.0 ? std::ceil((s.t_final - s.t) / s.dt) : 1.0, insts(b)[i].ntiles);
+    tiles += insts(b)[i].ntiles;
+  }
+  std::sort(left.begin(), left.end());
+  double steps = 1.0;
+  for (size_t i = 0; i < left.size() && 2 * tiles >= tiles_listed; ++i) {
+    steps = left[i].first;
+    tiles -= left[i].second;
+  }
+  const double r = std::floor(steps / b->graph_steps);
+  return r < 1.0 ? 1 : (r > 64.0 ? 64 : (int)r);
+}
+
 // Lay out the arena, upload every instance and prepare the device tables.
 alw_status build(alw_batch *b) {
   const int n = (int)b->pend.size();
@@ -575,10 +596,13 @@ alw_status autotune(alw_batch *b) {
       best = cands[i].t;
     }
   }
-  // A replay costs a read-back (about 15 us); steps captured beyond the last one still cost their launches, and each
-  // captured step its share of the graph's instantiation.  Measured (GB300, us per run at 2 / 4 / 8 / 32 steps): 6
-  // grids up to 160^2 1172 / 1133 / 1170 / 1369, 10 up to 300^2 1632 / 1561 / 1638 / 1673, 48 up to 512^2 (1600
-  // tiles) 5952 / 5924 / 6052 / 6610.
+  // Steps captured beyond the last one still cost their launches, and each captured step its share of the graph's
+  // instantiation; a read-back (about 15 us) follows the first replay of a work list and then only where it may be
+  // compacted (replays_ahead).  Microseconds per run (GB300) at 4 / 8 / 16 / 32 steps per graph, and at 4 with a
+  // read-back after every replay:
+  //   64 grids of 64^2, 11 steps    552 / 627 / 651 / 902; 567       153 steps   6253 / 6242 / 6187 / 6260; 6834
+  //   16 grids of 48^2-96^2, 410 steps                             16060 / 16717 / 17232 / 17297; 17172
+  //   48 grids of 64^2-512^2, 45 steps  3757 / 3785 / 4031 / 4419; 3842   417 steps  49940 / 51050 / 51180 / 51780; 50970
   best.steps_per_graph = total >= 4096 ? 2 : 4;
   best.grid_ctas = 0;  // occupancy cap
   b->tuning = best;
@@ -727,9 +751,9 @@ alw_status alw_batch_run(alw_batch *b, int64_t *replays_out) {
     st = build_graph(b, b->tuning.steps_per_graph, ntiles_now);
     if (st) return st;
     // replay until half of this work list is dead, then compact it
-    for (;;) {
-      B_CUDA(cudaGraphLaunch(b->graph, b->stream));
-      ++replays;
+    for (int ahead = 1;; ahead = replays_ahead(b, live, ntiles_now)) {
+      for (int r = 0; r < ahead; ++r) B_CUDA(cudaGraphLaunch(b->graph, b->stream));
+      replays += ahead;
       B_CUDA(cudaMemcpyAsync(b->h_state, b->d_state, sizeof(DevState) * ninst, cudaMemcpyDeviceToHost, b->stream));
       B_CUDA(cudaStreamSynchronize(b->stream));
       int live_tiles = 0, now_live = 0;

@@ -189,3 +189,19 @@ def test_batch_one_launch_per_stage_matches_per_hamiltonian_launches(tile_w):
     for inst, (a, sa), (c, sc) in zip(insts, outs[False], outs[True]):
         assert sa.t == sc.t == inst.t_final
         assert np.max(np.abs(a - c)) <= MIXED_SOLVE_TOL
+
+
+def test_end_times_far_apart():
+    # 4 to about 300 steps: several replays between read-backs, and the work list compacted twice
+    insts = [inputs.Instance(n, ham, 0.3 * n, t / math.pi**2)
+             for n, ham, t in ((40, "burgers2d", 0.1), (72, "negcos2d", 3.0), (33, "burgers2d", 0.5), (64, "burgers2d", 5.0))]
+    with native.Batch(precision="mixed") as b:
+        for inst in insts:
+            phi0, _ = inputs.instance_phi0(inst)
+            b.add(nx=inst.n, ny=inst.n, xlo=-2.0, xhi=2.0, ylo=-2.0, yhi=2.0, ham=inst.ham, phi0=phi0, t_final=inst.t_final)
+        b.set_tuning(steps_per_graph=4, tile_w=64)
+        b.run()
+        for k, inst in enumerate(insts):
+            ref, steps = _single(inst, "mixed", "arclength")
+            assert b.get_state(k).steps == steps and b.get_state(k).t == inst.t_final
+            np.testing.assert_array_equal(b.get_phi(k), ref)
