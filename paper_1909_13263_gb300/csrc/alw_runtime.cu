@@ -393,10 +393,25 @@ alw_status build_graph(alw_solver *s, int loop_mode, int nsteps, cudaGraphExec_t
   return ALW_OK;
 }
 
+// Host-side fault injection for tests: the value of an environment variable, 0 where it is not set.
+int test_env(const char *name) {
+  const char *e = std::getenv(name);
+  return e ? std::atoi(e) : 0;
+}
+
+// (ALW_TEST_STATE_ERR=b: the host sees error bits b in every state it reads; the device work is unchanged)
 alw_status read_state(alw_solver *s) {
   ALW_CUDA(cudaMemcpyAsync(s->h_st, s->st, sizeof(DevState), cudaMemcpyDeviceToHost, s->stream));
   ALW_CUDA(cudaStreamSynchronize(s->stream));
+  s->h_st->err |= test_env("ALW_TEST_STATE_ERR");
   return ALW_OK;
+}
+
+// The error bits of the state last read: 2 where a tile load or the barrier between stages gave up, 1 where a stage
+// met a non-finite dH/dp.
+alw_status state_error(const alw_solver *s) {
+  if (s->h_st->err & 2) return fail(ALW_ETIMEOUT, "a bounded device wait gave up at t = %.17g", s->h_st->t);
+  return s->h_st->err ? fail(ALW_ENONFINITE, "non-finite dH/dp detected at t = %.17g", s->h_st->t) : ALW_OK;
 }
 
 // Load interior values from a dense device array of doubles/floats into the current phi^n.
@@ -649,10 +664,7 @@ alw_status alw_set_phi0(alw_solver *s, const double *host_phi, size_t n) {
 // Host-side fault injection for the no-progress check of alw_step_to: with
 // ALW_TEST_FREEZE_STATE_AFTER=n (n >= 1) in the environment, the check sees the device state as it
 // was at its n-th read, as if the device had stopped advancing; the device work is unchanged.
-static int test_freeze_after() {
-  const char *e = std::getenv("ALW_TEST_FREEZE_STATE_AFTER");
-  return e ? std::atoi(e) : 0;
-}
+static int test_freeze_after() { return test_env("ALW_TEST_FREEZE_STATE_AFTER"); }
 
 alw_status alw_step_to(alw_solver *s, double t_final, int64_t *steps_out) {
   alw_status st = check_solver(s);
@@ -668,7 +680,7 @@ alw_status alw_step_to(alw_solver *s, double t_final, int64_t *steps_out) {
   st = read_state(s);
   if (st) return st;
   const int64_t steps0 = s->h_st->steps;
-  if (s->h_st->err) return fail(ALW_ENONFINITE, "non-finite dH/dp detected");
+  if ((st = state_error(s))) return st;
   s->h_tf[0] = t_final;
   ALW_CUDA(cudaMemcpyAsync(&s->st->t_final, s->h_tf, sizeof(double), cudaMemcpyHostToDevice, s->stream));
   int replays = 1, stalls = 0;
@@ -707,7 +719,7 @@ alw_status alw_step_to(alw_solver *s, double t_final, int64_t *steps_out) {
     }
     if (s->h_st->err) {
       if (steps_out) *steps_out = s->h_st->steps - steps0;
-      return fail(ALW_ENONFINITE, "non-finite dH/dp detected at t = %.17g", s->h_st->t);
+      return state_error(s);
     }
     if (s->h_st->steps - steps0 > 2000000000ll) return fail(ALW_ETIMEOUT, "step limit reached");
     const double rem = t_final - s->h_st->t;
@@ -760,8 +772,7 @@ alw_status alw_sync(alw_solver *s) {
   if (!s) return fail(ALW_EINVAL, "solver is NULL");
   alw_status st = read_state(s);
   if (st) return st;
-  if (s->h_st->err) return fail(ALW_ENONFINITE, "non-finite dH/dp detected");
-  return ALW_OK;
+  return state_error(s);
 }
 
 static alw_status gather_dense(alw_solver *s, int which, void *dst, int dtype) {

@@ -475,7 +475,7 @@ void worker_main(alw_server *s) {
       if (ds.t < ds.t_final && !ds.err) {
         keep.push_back(r);
       } else {
-        r->status = ds.err ? ALW_ENONFINITE : ALW_OK;
+        r->status = ds.err & 2 ? ALW_ETIMEOUT : ds.err ? ALW_ENONFINITE : ALW_OK;
         r->steps = ds.steps;
         r->steps_cur = ds.cur;
         done.push_back(r);

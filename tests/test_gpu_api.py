@@ -339,3 +339,19 @@ def test_gpu_reproduces_tables_1_2(ham, table, tf, factor, weights):
         ex = -np.cos(np.pi * (x - tf)) if ham == "advect1d" else exact.negcos_1d(ham, x, tf)
         e = np.abs(got - ex).max()
         assert tab[n][weights] / factor < e < tab[n][weights] * factor, (n, e, tab[n][weights])
+
+
+def test_lost_waits_are_reported_as_timeout(monkeypatch):
+    # host-side injection: error bit 2, which the kernels set when a bounded wait gave up, in the states the host reads
+    case = Case(2, 64, 48, "burgers2d", precision="mixed", lo=-2.0, hi=2.0)
+    with case.solver() as s:
+        s.set_phi0(case.field(seed=3, kind="smooth"))
+        for bits, status in ((2, native.ETIMEOUT), (3, native.ETIMEOUT), (1, native.ENONFINITE)):
+            monkeypatch.setenv("ALW_TEST_STATE_ERR", str(bits))
+            for call in (lambda: s.step_to(0.2), s.sync):
+                with pytest.raises(native.AlwError) as e:
+                    call()
+                assert e.value.status == status
+        monkeypatch.delenv("ALW_TEST_STATE_ERR")
+        s.step_to(0.2)
+        assert s.get_state().t == 0.2
