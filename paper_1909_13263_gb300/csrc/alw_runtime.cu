@@ -147,6 +147,7 @@ struct alw_solver {
   bool multi2d = false;     // 2D float grid: several steps per cooperative launch
   bool ghosts2d = false;    // the 2D float kernel extrapolates the ghosts (see Stage2DParams)
   SoloState *solo = nullptr;  // what their CTAs share
+  int many_launches = 0;    // counted for fault injection only
   bool use2d = false;       // persistent TMA kernel (2D float variants)
   int shape64 = 0;          // FP64 2D: tile shape (kShape64)
   CUtensorMap maps[6];      // tensor maps of the padded arrays (see Stage2DParams)
@@ -358,18 +359,29 @@ alw_status enqueue_step(alw_solver *s, int loop_mode) {
   return ALW_OK;
 }
 
+// Host-side fault injection for tests: the value of an environment variable, 0 where it is not set.
+int test_env(const char *name) {
+  const char *e = std::getenv(name);
+  return e ? std::atoi(e) : 0;
+}
+
 bool many_steps(const alw_solver *s) { return s->line64 || s->multi2d; }
 int graph_steps(const alw_solver *s) { return s->nx * (long long)s->ny >= (1 << 22) ? 4 : 16; }
 
 // Enqueue n RK3 steps in one launch (the 1D FP64 cluster, or a cooperative launch of the 2D float kernel).  Where
-// the device has no room for the cooperative grid at once (shared or partitioned GPUs), nothing is enqueued and
-// the solver turns to launches per stage.
+// the device has no room for the cooperative grid or the cluster at once, or takes neither (shared or partitioned
+// GPUs), nothing is enqueued and the solver turns to launches per stage.  (ALW_TEST_NO_ROOM_FROM=k, k >= 1: a solver's
+// k-th launch of this kind and later ones are refused so.)
 alw_status enqueue_many(alw_solver *s, int loop_mode, int n) {
   const StageParams p = make_params(s, 3, 3, loop_mode);
-  const int e = s->line64 ? launch_line64(p, n, s->stream) : launch_stage(s, p, n);
-  if (s->multi2d && e == (int)cudaErrorCooperativeLaunchTooLarge) {
+  const int refuse = test_env("ALW_TEST_NO_ROOM_FROM");
+  int e = (int)cudaErrorCooperativeLaunchTooLarge;
+  if (refuse <= 0 || ++s->many_launches < refuse)
+    e = s->line64 ? launch_line64(p, n, s->stream) : launch_stage(s, p, n);
+  if (e == (int)cudaErrorCooperativeLaunchTooLarge || e == (int)cudaErrorNotSupported ||
+      e == (int)cudaErrorInvalidClusterSize || e == (int)cudaErrorLaunchOutOfResources) {
     cudaGetLastError();
-    s->multi2d = false;
+    s->multi2d = s->line64 = false;
     return ALW_OK;
   }
   ALW_LAUNCH(e);
@@ -391,12 +403,6 @@ alw_status build_graph(alw_solver *s, int loop_mode, int nsteps, cudaGraphExec_t
   cudaGraphDestroy(g);
   if (e != cudaSuccess) return fail(ALW_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
   return ALW_OK;
-}
-
-// Host-side fault injection for tests: the value of an environment variable, 0 where it is not set.
-int test_env(const char *name) {
-  const char *e = std::getenv(name);
-  return e ? std::atoi(e) : 0;
 }
 
 // (ALW_TEST_STATE_ERR=b: the host sees error bits b in every state it reads; the device work is unchanged)

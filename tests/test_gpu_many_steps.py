@@ -118,3 +118,41 @@ def test_extrapolated_ghosts_match_oracle(shape, precision):
                 phi = s.get_stage_phi(stage) if stage < 3 else s.get_phi()
                 errs.append(rel_err(phi, ref[stage - 1]))
     assert max(errs) <= 64 * 2.0**-24, errs
+
+
+@pytest.mark.parametrize("first_refused", [1, 2, 3])
+@pytest.mark.parametrize("how", ["advance", "step_to"])
+@pytest.mark.parametrize("kind", ["mixed", "fp32", "line"])
+def test_no_room_for_many_steps_returns_to_single_stages(kind, how, first_refused, monkeypatch):
+    # a launch of whole steps is refused, at once or in the middle of a call: the stages run one by one from there on
+    if kind == "line":
+        case = Case(1, 200, 1, "burgers1d", alpha_mode="local_lagged")
+        phi0, steps = case.field(seed=4, kind="smooth"), 1200
+    else:
+        case = _case((127, 95), precision=kind)
+        phi0, steps = _phi0(case), 200
+    tf = None
+
+    def solve():
+        with case.solver() as s:
+            s.set_phi0(phi0)
+            if how == "advance" or tf is None:
+                s.advance(steps)
+            else:
+                s.step_to(tf)
+            phi, st = s.get_phi(), s.get_state()
+            s.advance(3)
+            s.step_to(s.get_state().t * 1.01)
+            s.sync()
+            return phi, st.t, st.steps
+
+    tf = solve()[1]
+    ref = solve()
+    monkeypatch.setenv("ALW_TEST_NO_ROOM_FROM", str(first_refused))
+    got = solve()
+    if kind == "line":   # the cluster kernel and the stage kernel round differently
+        assert got[1] == pytest.approx(ref[1], rel=1e-12) and abs(got[2] - ref[2]) <= 1
+        assert rel_err(got[0], ref[0]) <= 1e-12
+    else:
+        assert got[1:] == ref[1:]
+        np.testing.assert_array_equal(got[0], ref[0])
