@@ -64,7 +64,6 @@ __global__ void __launch_bounds__(kLineThreads) line64_kernel(const __grid_const
   __shared__ int s_nrare[2];
   __shared__ double s_wmax[3][kLineThreads / 32];     // maximum of |dH/dp| per stage and warp
   __shared__ double s_alpha;                          // the grid's, of the last stage
-  __shared__ int s_phase[3], s_broken;                // stages closed (checked against the neighbours')
 
   double t = st->t, dt = st->dt;
   const double t_final = st->t_final;
@@ -74,9 +73,7 @@ __global__ void __launch_bounds__(kLineThreads) line64_kernel(const __grid_const
   double *P = reinterpret_cast<double *>(p.out0);
   for (int k = tid; k < count + 6; k += blockDim.x) s_phi[0][k] = P[GX + first + k - 3];
   if (tid < 2) s_nrare[tid] = 0;
-  if (tid == 0) s_broken = 0;
   const int warps = blockDim.x / 32;
-  int phase = 0;
   const bool local_alpha = p.alpha_mode == A_LOCAL_LAGGED || p.alpha_mode == A_LOCAL_EXACT;
   cluster_barrier();
 
@@ -173,27 +170,19 @@ __global__ void __launch_bounds__(kLineThreads) line64_kernel(const __grid_const
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) ax = max_bits(ax, __shfl_xor_sync(0xffffffffu, ax, o));
       if (lane == 0) s_wmax[stage - 1][tid >> 5] = ax;
-      if (tid == 0) s_phase[stage - 1] = ++phase;
       cluster_barrier();
-      // ---- the first warp: the maximum over the cluster's warps, and a check that all CTAs closed this stage
+      // ---- the first warp: the maximum over the cluster's warps
       if (tid < 32) {
         double a = 0.0;
-        bool same = true;
-        for (int k = lane; k < ranks * warps && !s_broken; k += 32)
+        for (int k = lane; k < ranks * warps; k += 32)
           a = max_bits(a, cl.map_shared_rank(s_wmax[stage - 1], k / warps)[k % warps]);
-        const int mine = s_phase[stage - 1];
-        if (lane < ranks && !s_broken) same = *cl.map_shared_rank(&s_phase[stage - 1], lane) == mine;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) a = max_bits(a, __shfl_xor_sync(0xffffffffu, a, o));
-        same = __all_sync(0xffffffffu, same);
-        if (lane == 0) {
-          s_alpha = a;
-          if (!same) s_broken = 1;
-        }
+        if (lane == 0) s_alpha = a;
       }
       // ---- ghost cells: from the neighbours (periodic images), or extrapolated at the grid's ends
       const int gt = tid - (blockDim.x - 32);   // by the last warp
-      if (gt >= 0 && gt < 6 && !s_broken) {
+      if (gt >= 0 && gt < 6) {
         const int g = gt < 3 ? first - 1 - gt : first + count + gt - 3;   // grid position
         const int cell = g - first + 3;
         if (p.bc == BC_PERIODIC || (g >= 0 && g < n)) {
@@ -240,7 +229,7 @@ __global__ void __launch_bounds__(kLineThreads) line64_kernel(const __grid_const
       st->alpha_bits[1][0] = double_to_bits(alpha2);
       st->alpha_bits[2][0] = double_to_bits(alpha);
     }
-    if (err || s_broken) st->err |= s_broken ? 2 : 1;
+    if (err) st->err |= 1;
   }
   cluster_barrier();  // no CTA leaves while another may still read its shared memory
 }
