@@ -44,50 +44,8 @@ enum { A_LOCAL_LAGGED = 0, A_LOCAL_EXACT = 1, A_GLOBAL_LAGGED = 2, A_GLOBAL_EXAC
 template <typename T> struct Arith;
 
 template <> struct Arith<double> {
-  // F(u) = u s + asinh(u) and s = sqrt(1+u^2), with asinh|u| = log(|u| + s) reusing s.  F only
-  // enters divided differences (F(b) - F(a)) / (b - a) over intervals longer than 1e-3 s, so
-  // its absolute error is what counts: log of the rounded |u| + s >= 1 errs by about one unit
-  // of 1, like a correctly rounded F of size one.
-  __device__ __forceinline__ static void F(double u, double &Fu, double &s) {
-    s = sqrt(fma(u, u, 1.0));
-    Fu = fma(u, s, copysign(log(fabs(u) + s), u));
-  }
-  // mean of sqrt(1+u^2) over [a, b]; near a == b the divided difference is 0/0, so its Taylor
-  // series about the midpoint is summed instead (below 1e-3 of the mean of the end values
-  // sa, sb, which bounds sqrt(1 + m^2) from above; both forms are accurate near the switch).
-  __device__ __forceinline__ static double G(double a, double Fa, double sa, double b, double Fb, double sb) {
-    const double h = b - a;
-    if (fabs(h) > 5e-4 * (sa + sb)) return (Fb - Fa) / (2.0 * h);
-    const double m = 0.5 * (a + b);
-    const double s2 = fma(m, m, 1.0), s = sqrt(s2);
-    const double r = 1.0 / s2, m2 = m * m, h2 = h * h;
-    // f'' = s2^{-3/2}, f'''' = (12 m^2 - 3) s2^{-7/2}, f^(6) = (45 - 540 m^2 + 360 m^4) s2^{-11/2}
-    const double f2 = r / s;
-    const double f4 = (12.0 * m2 - 3.0) * r * r * r / s;
-    const double f6 = (45.0 - 540.0 * m2 + 360.0 * m2 * m2) * r * r * r * r * r / s;
-    return s + h2 * (f2 / 24.0 + h2 * (f4 / 1920.0 + h2 * f6 / 322560.0));
-  }
-  // nonlinear weights (Eq. WLOC1): returns omega_0, omega_2 from q_k = (eps + beta_k)^2 in the
-  // product form omega_k = d_k prod_{l != k} q_l / sum_m d_m prod_{l != m} q_l (one division;
-  // the quotients d_k / q_k of Eq. WLOC1 when the products leave the double range)
-  __device__ __forceinline__ static void weights(double q0, double q1, double q2, double &w0, double &w2) {
-    const double n0 = 0.1 * (q1 * q2), n2 = 0.3 * (q0 * q1);
-    const double den = fma(0.6, q0 * q2, n0 + n2);
-    if (den > 1e-290 && den < 1e290) {
-      const double r = 1.0 / den;
-      w0 = n0 * r;
-      w2 = n2 * r;
-    } else {
-      const double a0 = 0.1 / q0, a1 = 0.6 / q1, a2 = 0.3 / q2;
-      const double sum = a0 + a1 + a2;
-      w0 = a0 / sum;
-      w2 = a2 / sum;
-    }
-  }
   __device__ __forceinline__ static double cosv(double x) { return cos(x); }
   __device__ __forceinline__ static double sinv(double x) { return sin(x); }
-  __device__ __forceinline__ static double sqrtv(double x) { return sqrt(x); }
-  __device__ __forceinline__ static double rcp(double x) { return 1.0 / x; }
 };
 
 template <> struct Arith<float> {
@@ -125,8 +83,6 @@ template <> struct Arith<float> {
   }
   __device__ __forceinline__ static float cosv(float x) { return __cosf(x); }
   __device__ __forceinline__ static float sinv(float x) { return __sinf(x); }
-  __device__ __forceinline__ static float sqrtv(float x) { return sqrtf(x); }
-  __device__ __forceinline__ static float rcp(float x) { return __frcp_rn(x); }
 };
 
 // --------------------------------------------------------------------------
@@ -212,20 +168,17 @@ __device__ __forceinline__ void weno_sweep(const T (&v)[K + 5], T rdx, T dx, T e
 }
 
 // --------------------------------------------------------------------------
-// Hamiltonians (runtime kind, uniform across the grid).
+// Hamiltonians (runtime kind, uniform across the grid): the 1D kinds in float, and in double the kinds that
+// ham_node64 (alw_node64.cuh) leaves to these; the 2D float stages have theirs in alw_stage2d.cuh.
 
 // (x, y) is the node's position; only Example 11's H depends on it.
 template <typename T>
 __device__ __forceinline__ T ham_value(int kind, T p, T q, T x, T y) {
   using A = Arith<T>;
   switch (kind) {
-    case H_BURGERS2D: { const T z = p + q + T(1); return T(0.5) * z * z; }
-    case H_NEGCOS2D: return -A::cosv(p + q + T(1));
-    case H_SIN2D: return A::sinv(p + q);
     case H_ADVECT1D: return p;
     case H_BURGERS1D: { const T z = p + T(1); return T(0.5) * z * z; }
     case H_NEGCOS1D: return -A::cosv(p + T(1));
-    case H_EIKONAL2D: return A::sqrtv(p * p + q * q + T(1));
     case H_NONCONVEX1D: return T(0.25) * (p * p - T(1)) * (p * p - T(4));
     case H_OPTCTRL2D: {
       // sin(y) p + (sin(x) + sign q) q - sin^2(y)/2 - (1 - cos x), with (sign q) q = |q|
@@ -242,36 +195,9 @@ template <typename T>
 __device__ __forceinline__ void node_alpha(int kind, T um, T up, T vm, T vp, T x, T y, T &ax, T &ay) {
   using A = Arith<T>;
   switch (kind) {
-    case H_BURGERS2D: {
-      const T a = fabs(um + vm + T(1)), b = fabs(um + vp + T(1)), c = fabs(up + vm + T(1)), d = fabs(up + vp + T(1));
-      ax = ay = fmax(fmax(a, b), fmax(c, d));
-    } break;
-    case H_NEGCOS2D: {
-      const T a = fabs(A::sinv(um + vm + T(1))), b = fabs(A::sinv(um + vp + T(1)));
-      const T c = fabs(A::sinv(up + vm + T(1))), d = fabs(A::sinv(up + vp + T(1)));
-      ax = ay = fmax(fmax(a, b), fmax(c, d));
-    } break;
-    case H_SIN2D: {
-      const T a = fabs(A::cosv(um + vm)), b = fabs(A::cosv(um + vp));
-      const T c = fabs(A::cosv(up + vm)), d = fabs(A::cosv(up + vp));
-      ax = ay = fmax(fmax(a, b), fmax(c, d));
-    } break;
     case H_ADVECT1D: ax = T(1); ay = T(0); break;
     case H_BURGERS1D: ax = fmax(fabs(um + T(1)), fabs(up + T(1))); ay = T(0); break;
     case H_NEGCOS1D: ax = fmax(fabs(A::sinv(um + T(1))), fabs(A::sinv(up + T(1)))); ay = T(0); break;
-    case H_EIKONAL2D: {
-      T mx = T(0), my = T(0);
-      const T us[2] = {um, up}, vs[2] = {vm, vp};
-#pragma unroll
-      for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          const T r = A::rcp(A::sqrtv(us[a] * us[a] + vs[b] * vs[b] + T(1)));
-          mx = fmax(mx, fabs(us[a]) * r);
-          my = fmax(my, fabs(vs[b]) * r);
-        }
-      ax = mx; ay = my;
-    } break;
     case H_NONCONVEX1D: {
       // H_p = p^3 - 5p/2; interior extrema of H_p at p = +-sqrt(5/6), where |H_p| = (5/3) sqrt(5/6)
       const T lo = fmin(um, up), hi = fmax(um, up);
