@@ -169,3 +169,30 @@ def test_tiles_of_noise_match_oracle(nx, ny, weights):
     scattered = np.random.default_rng(9).random((ny - ny // 2, nx)) < 0.05
     phi0[ny // 2:][scattered] += 0.1 * rough[ny // 2:][scattered]
     assert max(_errors(case, phi0)) <= FP64_TOL
+
+
+# What the launches of whole steps leave behind (field, ghosts, grid maxima) is what single stages go on from: three
+# steps in one launch and one by stages, against four by stages with the same time steps.
+@pytest.mark.parametrize("nx", [5, 64, 200, 1024])
+@pytest.mark.parametrize("kw", [dict(bc="periodic"), dict(bc="linextrap", alpha_mode="global_lagged"),
+                                dict(bc="linextrap", weights="jp", alpha_mode="fixed", alpha_fixed=(5.0, 0.0))],
+                         ids=lambda k: "-".join(map(str, k.values())))
+def test_stages_go_on_from_a_line_launch(nx, kw):
+    case = Case(1, nx, 1, "burgers1d", **{"alpha_mode": "local_lagged", **kw})
+    x, _ = inputs.axis(nx, -1.0, 1.0, case.bc)
+    phi0 = -np.cos(np.pi * x + 0.3) + 0.2 * np.abs(x)
+
+    def stages(s):
+        a = case.alpha_fixed if case.alpha_mode == "fixed" else s.get_state().alpha
+        for stage in (1, 2, 3):
+            s.run_stage(stage, 0.6 * case.dx / a[0])
+
+    with case.solver() as s, case.solver() as r:
+        s.set_phi0(phi0)
+        s.advance(3)
+        stages(s)
+        r.set_phi0(phi0)
+        for _ in range(4):
+            stages(r)
+        assert rel_err(s.get_phi(), r.get_phi()) <= FP64_TOL
+        assert s.get_state().alpha[0] == pytest.approx(r.get_state().alpha[0], rel=FP64_TOL)
