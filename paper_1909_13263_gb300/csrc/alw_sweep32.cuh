@@ -507,10 +507,12 @@ __device__ __forceinline__ int sweep_stream_near(LoadV v_at, V rdx, V e1, V size
     V nk1, qm1, qp1;
     stencil(p + 1, nk1, qm1, qp1);
     const V am = vmul(nk, qm), ap = vmul(nk1, qp1);       // what is added to lin^- and lin^+
-    const V s0 = vfma(c(-0.2f), vadd(W[p + 2], W[p + 3]),
-                      vfma(c(1.0f / 30.0f), vadd(W[p + 1], W[p + 4]), vadd(v[p + 2], v[p + 3])));
+    // the small terms among themselves first: added to the large sum one by one, those below half its last place are
+    // lost at every node alike (8192^2 Example 3: H high by 3e-8 on average, 6.6e-9 of phi at t = 0.05; so 1.0e-9)
+    const V small = vfma(c(1.0f / 30.0f), vadd(W[p + 1], W[p + 4]),
+                         vfma(c(-0.2f), vadd(W[p + 2], W[p + 3]), vadd(ap, am)));
     const V d0 = vfma(c(-2.0f), T[p + 3], vadd(T[p + 2], T[p + 4]));   // (lin^+ - lin^-) 30
-    emit(p, vadd(s0, vadd(ap, am)), vfma(c(1.0f / 30.0f), d0, vsub(ap, am)));
+    emit(p, vadd(vadd(v[p + 2], v[p + 3]), small), vfma(c(1.0f / 30.0f), d0, vsub(ap, am)));
     nk = nk1;
     qm = qm1;
   }

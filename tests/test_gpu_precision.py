@@ -5,6 +5,8 @@ import numpy as np
 import pytest
 
 import exact
+import oracle
+from gpucase import Case
 from paper_1909_13263_gb300 import inputs, native
 
 pytestmark = pytest.mark.gpu
@@ -58,3 +60,20 @@ def test_burgers_hamiltonian_is_unbiased_on_constants(precision, alpha_mode):
         err = np.abs(s.get_phi() - (value - steps * dt / 2)).max()
     unit = dt / 2 if precision == "mixed" else value
     assert err <= steps * unit * 2.0**-24
+
+
+# The rounding of a smooth H must not lean to one side: over a line of 8192 nodes the mean error of L, from the first
+# stage's increment against the oracle, stays below a tenth of the last place of the derivatives' sum (2^-22 for sums
+# up to 4, here pi); errors that fall at random average to a hundredth.
+@pytest.mark.parametrize("theta", [0.0, 0.3, 1.1, 2.0])
+def test_mixed_rounding_of_smooth_data_is_unbiased(theta):
+    case = Case(2, 8192, 32, "burgers2d", precision="mixed", lo=-2.0, hi=2.0, alpha_mode="fixed", alpha_fixed=(2.5, 2.5))
+    x, _ = inputs.axis(8192, -2.0, 2.0, "periodic")
+    phi = np.tile(-np.cos(0.5 * math.pi * x + theta), (32, 1))
+    dt = 2.0**-13
+    with case.solver() as s:
+        s.set_phi0(phi)
+        s.run_stage(1, dt)
+        L = (s.get_stage_phi(1) - s.get_phi()) / dt
+    err = L - oracle.L_of(case.cfg(), phi, np.array([2.5, 2.5]))
+    assert abs(err.mean()) <= 0.1 * 2.0**-22
