@@ -99,7 +99,7 @@ enum { ALW_DT_CFL = 0, ALW_DT_DX53 = 1 };
 
 /* Arithmetic.  FP64: all in double, except that on resolved data the small deviation of the nonlinear weights
  * from the linear ones is formed in float pairs (at least 44 significant bits) where its rounding stays below a
- * sixteenth of the last place of phi.  FP32: phi and all arithmetic in float.
+ * quarter of the last place of phi.  FP32: phi and all arithmetic in float.
  * MIXED: stencil arithmetic in float; phi^n is held as an unevaluated sum of
  * two floats (hi + lo, about 48 significant bits) and the RK stages store
  * float increments that carry the low part, lo + (phi_s - phi^n), so a stage

@@ -238,7 +238,7 @@ template <int W>
 int launch(const StageParams &p, int nsteps, cudaStream_t s) {
   LineParams q;
   q.p = p;
-  q.c = make_sweep64<W>(p.dx, p.eps);
+  q.c = make_sweep64<W>(p.dx, p.eps, p.nx);
   q.nsteps = nsteps;
   int ranks = 1;
   while (ranks < kLineCluster && p.nx > ranks * kLineNodes) ranks *= 2;

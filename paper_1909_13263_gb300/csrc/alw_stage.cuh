@@ -17,8 +17,8 @@ template <int PREC, int W>
 static SweepArgs<PREC> sweep_args(const StageParams &p) {
   SweepArgs<PREC> a;
   if constexpr (PREC == P_F64) {
-    a.c[0] = make_sweep64<W>(p.dx, p.eps);
-    a.c[1] = p.dim == 2 ? make_sweep64<W>(p.dy, p.eps) : a.c[0];
+    a.c[0] = make_sweep64<W>(p.dx, p.eps, p.nx);
+    a.c[1] = p.dim == 2 ? make_sweep64<W>(p.dy, p.eps, p.ny) : a.c[0];
   }
   return a;
 }

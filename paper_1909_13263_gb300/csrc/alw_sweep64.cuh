@@ -11,19 +11,21 @@
 // V = A2 - A1 and den = A0 + 6 A1 + 3 A2.  The linear part, which carries the accuracy of phi, stays
 // in double; the deviation is a weight error (w - d) times third differences T, and is formed in unevaluated
 // float pairs (df).  Its error, measured against 128-bit arithmetic on smooth, kinked and noisy data, is at
-// most 2^-46.5 |T|.  A node takes this form when |T| 2^10 (in units of phi) is at most |phi|, so that its error over
-// a stage, 2^-46.5 |T| cfl, is below 2^-57 |phi|, a sixteenth of phi's last place.
+// most 2^-46.5 |T|.  A node takes this form when |T| (in units of phi) times 2 n, n the nodes along the line (at least
+// 128), is at most |phi|: the derivative's error, 2^-46.5 |T| / dx, is then at most 2^-47.5 of the slope |phi| over
+// the line's length on every grid, and that of phi over a stage below 2^-55 |phi| / (n / 128).
 // Next to a kink T is as large as the jump and that fails, but there the weights of the stencils that
 // cross the kink nearly vanish.  The node is then expanded about its dominant candidate k,
 //   phi^- = phi^{-,k} + sum over the others of w_l (phi^{-,l} - phi^{-,k}),
 // with the candidate in double and the sum in pairs, if the terms of the sum meet the bound (their sizes
-// times 2^9, Jiang-Peng 2^10, at most |phi|).
+// times n, Jiang-Peng 2 n, at most |phi|).
 // Nodes that fail both (noise, data the grid does not resolve) are computed in double, side by side or, where a
 // tile holds many, segment by segment with each stencil's indicators shared by the two sides it serves.
 // The error of the one-sided derivatives against extended precision, as a share of that with double-precision
 // indicators (1000 lines of 40 to 1040 nodes each with sharp kinks, rounded corners or steep slopes): rms 0.68-0.79,
-// largest 0.19-0.86.  With 2^8, 2^7 and 2^8 for the three limits the largest were up to 4 times as large as the double
-// sweep's at kinks, and up to 14 times on finer grids.
+// largest 0.15-0.91; up to 4000 nodes rms 0.65-0.80, largest 0.61-1.4.  (With limits 2^8, 2^7 and 2^8 on every grid the
+// largest were up to 4 and 14 times the double sweep's.  With 2^10, 2^9 and 2^10 they were as good up to 1040 nodes, but
+// coarse grids paid: N = 320 through the kink 20.8 ms against 19.2, 16.7 with the first limits.)
 //
 // Arc-length indicators: with sigma = sqrt(1 + a^2) + sqrt(1 + b^2), h = b - a and t = h / sigma (= tanh of
 // half the difference of asinh b and asinh a), the mean of sqrt(1 + u^2) over [a, b], (F(b) - F(a)) / (2 h)
@@ -183,11 +185,11 @@ struct Sweep64 {
   double rdx, dx, eps_d;  // for the double form and the dominant-candidate form
   df scale;               // second differences of phi to the units of the indicators
   df eps;                 // arc length: 4 eps / dx^2; Jiang-Peng: eps
-  float t2phi;            // 2^10 T in units of phi
+  float t2phi;            // 2 n T in units of phi, n >= 128
 };
 
 template <int W>
-inline Sweep64 make_sweep64(double dx, double eps) {
+inline Sweep64 make_sweep64(double dx, double eps, int n) {
   auto pair = [](double x) {
     df r;
     r.h = (float)x;
@@ -208,7 +210,7 @@ inline Sweep64 make_sweep64(double dx, double eps) {
   c.cdev = arc ? dx / 20.0 : 0.05 / 32.0;
   c.scale = pair(arc ? rdx * rdx : 32.0 * rdx);
   c.eps = pair(arc ? 4.0 * eps * rdx * rdx : 1024.0 * eps);
-  c.t2phi = (float)(1024.0 * (arc ? dx * dx : dx / 32.0));
+  c.t2phi = (float)((n > 128 ? 2.0 * n : 256.0) * (arc ? dx * dx : dx / 32.0));
   return c;
 }
 

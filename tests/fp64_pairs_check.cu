@@ -61,7 +61,7 @@ struct Sum {
 template <int W>
 static void line(const std::vector<double> &p, double dx, double eps, Sum &r) {
   typedef long double L;
-  const Sweep64 c = make_sweep64<W>(dx, eps);
+  const Sweep64 c = make_sweep64<W>(dx, eps, (int)p.size() - 6);
   for (int i = 0; i + 6 < (int)p.size(); ++i) {
     double d[2] = {0, 0};
     const double *a = &p[i];
