@@ -603,7 +603,8 @@ def bench_fp64(args, stream):
         ms = e0.elapsed_time(e1) / args.fp64_steps
     return {"workload": f"ex3_burgers2d_{n}sq", "value": n * n / (ms * 1e-3), "unit": UNIT, "ms_per_step": ms,
             "steps": args.fp64_steps, "bound": "fp64 pipe",
-            "fp64_pipe_note": "56 FP64 operations per node and stage; ncu at 2048^2: FP64 pipe 80 % busy"}
+            "fp64_pipe_note": "59-63 FP64 operations per node and stage; ncu at 2048^2: FP64 pipe 84 % of its peak "
+                              "(profiles/stage_kernel_fp64_ex3_arclength_2048.md)"}
 
 
 def run_ours(args):
@@ -774,7 +775,7 @@ def run_ours(args):
         "dtype": "f32" if args.precision != "fp64" else "f64", "data": "synthetic",
         "config": {"workload": f"ex3_burgers2d_{n}sq", "nx": n, "ny": n, "precision": args.precision,
                    "weights": args.weights, "hamiltonian": "(p+q+1)^2/2", "alpha": "global_lagged",
-                   "step": "one TVD-RK3 step (3 fused stage kernels)",
+                   "step": "one TVD-RK3 step (3 fused stages; float grids run several steps per cooperative launch)",
                    "l2": "inputs larger than L2 (no flush)", "parallelism": f"replicas{ws}"},
         "roofline": roof,
         "cpu_baseline": cpu,

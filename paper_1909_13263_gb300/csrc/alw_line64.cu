@@ -11,9 +11,9 @@
 // node before, which is handed over in shared memory (alw_sweep64.cuh has the arithmetic).
 //
 // What bounds it: the latency of one stage's dependent operations.  Measured (GB300, RK3 steps of Example 6):
-// N = 80 smooth 13 us per step (three stages), with kinks 20-43 us, against 72 us for the same arithmetic in one
+// N = 80 smooth 13 us per step (three stages), with kinks 20-68 us, against 72 us for the same arithmetic in one
 // launch per stage (rare nodes included) and 570 us for the double-precision indicators; whole solves N = 80
-// to t = 0.5/pi^2 8.1 -> 0.29 ms, N = 320 to 3.5/pi^2 195 -> 17 ms.
+// to t = 0.5/pi^2 8.1 -> 0.28 ms, N = 320 to 3.5/pi^2 195 -> 19.2 ms.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 

@@ -27,8 +27,13 @@
 // What bounds it: instruction issue and the FMA pipe from about 2048^2 up, one tile's latency and the grid barrier
 // below.  64 x 32 tiles with 8-node segments keep the work repeated at segment ends and the halo reads small with
 // two CTAs (16 warps) per SM.  Measured (GB300, us per RK3 step of Example 3, MIXED; against a staged differences
-// pass, the short-interval sweep and a launch per stage): 8192^2 1174 -> 996 alone, a pass of ten steps 13.31 ->
-// 11.58 ms; 403 x 397 to t = 0.5/pi^2 2633 -> 1684 us; FP32 2048^2, forty steps 5314 -> 3033 us.
+// pass, the short-interval sweep and a launch per stage): 8192^2 1174 -> 988 alone, a pass of ten steps 13.31 ->
+// 11.47 ms; 403 x 397 to t = 0.5/pi^2 2633 -> 1689 us; FP32 2048^2, forty steps 5314 -> 3074 us.  Slower than it was:
+// FP32 with a trigonometric Hamiltonian on grids so fine that all segments sweep in full (Example 10, 4096^2 465 ->
+// 489, 8192^2 1746 -> 1842): there the handover of the column sweep's results through shared memory gains nothing
+// (the near-linear form tried in vain is below 1 % of it); and launches of single stages on grids of a few tiles
+// with kinks, where a tile waits for the near-linear form and then for its list (a batch of 16 grids of 48^2-96^2, 410
+// steps, 14.4 -> 16.1 ms).
 #pragma once
 #include <type_traits>
 

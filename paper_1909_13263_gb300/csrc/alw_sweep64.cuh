@@ -38,10 +38,11 @@
 // The loop over a segment's nodes is rolled and one code serves both directions: unrolled, the sweeps did not
 // fit the instruction cache (2.1 stall cycles per issue waiting for instructions).
 //
-// Measured (GB300, RK3 steps of Example 3, against the sweep with double indicators): 2048^2 18.6 -> 1.53 ms per
-// step, 400^2 1570 -> 99 us; Example 10 on 1024^2 (kinks, double sine and cosine) 8.4 -> 0.81 ms.  On smooth
-// data (cosine, dx = 0.1 to 5e-4) the error of the one-sided derivatives is 0.9-1.3e-16 rms against 0.9-1.8e-16.
-// What bounds it: the FP64 pipe, 56 operations per node (28 cycles of an SM; 80 % busy at 2048^2).
+// Measured (GB300, RK3 steps of Example 3, against the sweep with double indicators): 2048^2 18.4 -> 1.47 ms per
+// step, 400^2 1570 -> 97 us; Example 10 on 1024^2 (kinks, double sine and cosine) 8.33 -> 0.86 ms.  On smooth data
+// (cosine, dx = 0.1 to 5e-4) the error of the one-sided derivatives is 0.9-1.3e-16 rms against 0.9-1.8e-16.  Noise on
+// every node, where all of it ends in double: 2048^2 15.0 -> 16.6 ms (Jiang-Peng 5.0 -> 5.7), 512^2 the same.
+// What bounds it: the FP64 pipe, 59-63 operations per node and stage (30 cycles of an SM; 84 % of its peak at 2048^2).
 #pragma once
 #include <string.h>
 
