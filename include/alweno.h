@@ -183,10 +183,12 @@ alw_status alw_set_phi0(alw_solver *s, const double *host_phi, size_t n);
 alw_status alw_set_phi0_device(alw_solver *s, const void *dev_phi, int32_t dtype, size_t n);
 
 /* Advance to t_final with TVD-RK3 (Step 5): whole steps, the last one clipped.
- * Work is enqueued as CUDA-graph replays on the solver's stream; the call
- * returns after the device reports t >= t_final.  steps_out (nullable) gets
- * the number of steps taken by this call.  ALW_ENONFINITE if dH/dp became
- * non-finite (phi is left at the step where it was detected). */
+ * Work is enqueued on the solver's stream, as launches of many steps (1D FP64
+ * grids of up to 1024 nodes, 2D float grids; lagged or fixed alpha) or CUDA-graph
+ * replays; the call returns after the device reports t >= t_final.  steps_out
+ * (nullable) gets the number of steps taken by this call.  ALW_ENONFINITE if dH/dp
+ * became non-finite (phi is left at the step where it was detected), ALW_ETIMEOUT
+ * if a bounded device wait gave up or nothing advances. */
 alw_status alw_step_to(alw_solver *s, double t_final, int64_t *steps_out);
 
 /* Advance exactly nsteps TVD-RK3 steps (Step 5) with the CFL time step of
@@ -202,7 +204,8 @@ alw_status alw_advance(alw_solver *s, int64_t nsteps);
 alw_status alw_run_stage(alw_solver *s, int32_t stage, double dt);
 
 /* Wait for the solver's stream (no counterpart in the paper); returns
- * ALW_ENONFINITE if a stage flagged a non-finite dH/dp. */
+ * ALW_ENONFINITE if a stage flagged a non-finite dH/dp, ALW_ETIMEOUT if a bounded
+ * device wait gave up. */
 alw_status alw_sync(alw_solver *s);
 
 /* Copy the solution phi(x, t) of Eq. HJ at the solver's current time
